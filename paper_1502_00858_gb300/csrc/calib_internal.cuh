@@ -186,6 +186,19 @@ cudaError_t launch_tcg_step(const LMArgs& a, bool last, cudaStream_t s);
 cudaError_t launch_rtr_eval(const LMArgs& a, int mode, cudaStream_t s);
 cudaError_t launch_hv_output(const LMArgs& a, float* out, cudaStream_t s);
 
+// ---- the whole J-update of an agent in one CTA (jupdate.cu)
+constexpr int JUPDATE_SMEM_MAX = 220 * 1024;
+struct JUpdateArgs {
+    const float2* U; const float2* S;  // statistics, full circulant layout
+    int* status;
+    int n_lm, n_cg;
+    int threads, chunk;  // threads a CTA, diagonals summed at a time
+};
+bool jupdate_plan(int N, int K, int A, int sms, JUpdateArgs& q);  // false: the separate kernels
+cudaError_t prepare_jupdate_kernels();
+// mode: LM_BEGIN_FROM_PARTIALS or LM_BEGIN_REUSE (LMEvalMode)
+cudaError_t launch_jupdate(const LMArgs& a, const JUpdateArgs& q, bool rtr, int mode, cudaStream_t s);
+
 // ---- launchers (sage.cu): the SAGE decomposition of the J-update over directions (step D1)
 struct SageArgs {
     const float2* U; const float2* S;       // statistics of all directions (full circulant layout)

@@ -109,13 +109,16 @@ struct calib_ctx {
     std::vector<int> slot_h, slot_b_h;
     long long int_v = 0, int_c = 0;             // internal totals (float2)
     long long int_u = 0, int_s = 0;             // sufficient-statistics totals (float2)
-    double alg_bytes[8] = {0, 0, 0, 0, 0, 0, 0, 0};  // algorithmic bytes per launch of each profiled kind
-    double alg_flops[8] = {0, 0, 0, 0, 0, 0, 0, 0};  // algorithmic real flops per launch of each profiled kind
+    double alg_bytes[9] = {};  // algorithmic bytes per launch of each profiled kind
+    double alg_flops[9] = {};  // algorithmic real flops per launch of each profiled kind
     std::vector<uint8_t> flags_h;
 
     // device
     float2 *V = nullptr, *C = nullptr, *ssU = nullptr, *ssS = nullptr;
     int formulation = 0;  // 0 sufficient statistics, 1 direct
+    // small problems in the statistics form, LM or RTR: the J-update in one launch (jupdate.cu)
+    bool one_launch = false;
+    JUpdateArgs jup{};
     bool ss_dirty = true;
     DiagDesc* desc = nullptr;
     int *slot = nullptr, *slot_b = nullptr, *T_d = nullptr;
@@ -162,10 +165,10 @@ struct calib_ctx {
     long long launches = 0;
     bool profiling = false;
     // 4 sweep kinds, the PCG step, the LM evaluation, the statistics pass, the fusion-centre step
-    // (gauge, Z-update, Y-update and records of one iteration, timed together)
-    static constexpr int PROF_KINDS = 8;
-    double prof_ms[PROF_KINDS] = {0, 0, 0, 0, 0, 0, 0, 0};
-    long long prof_n[PROF_KINDS] = {0, 0, 0, 0, 0, 0, 0, 0};
+    // (gauge, Z-update, Y-update and records of one iteration, timed together), the one-launch J-update
+    static constexpr int PROF_KINDS = 9;
+    double prof_ms[PROF_KINDS] = {};
+    long long prof_n[PROF_KINDS] = {};
 };
 
 namespace {
@@ -482,6 +485,9 @@ int build_layout(calib_ctx* c, const uint8_t* flags) {
     for (int i = 0; i < 4; ++i) c->alg_flops[i] = flo[i];
     c->alg_bytes[6] = alg_stp;
     c->alg_flops[6] = flo_stp;
+    // one J-update: every pass's flops, the statistics read once for it
+    c->alg_bytes[8] = alg_sst;
+    c->alg_flops[8] = c->n_lm * (c->n_cg * flo[2] + flo[3]);
     c->TT_res = sweep_tile_samples(smax, K, false);
     c->TT_hv = sweep_tile_samples(smax, K, true);
     if (sweep_threads(smax) > 512) return fail(CALIB_EINVAL, "too many stations for one CTA per diagonal");
@@ -593,6 +599,17 @@ struct Enq {
         ok(c->jupdate == CALIB_JUPDATE_RTR ? launch_rtr_eval(la, mode, c->stream) : launch_lm_eval(la, mode, c->stream));
         end(pp);
     }
+    void jupdate(const LMArgs& la, int mode) {
+        ProfPair pp = begin(8);
+        JUpdateArgs ja = c->jup;
+        ja.U = c->ssU;
+        ja.S = c->ssS;
+        ja.status = c->status;
+        ja.n_lm = c->n_lm;
+        ja.n_cg = c->n_cg;
+        ok(launch_jupdate(la, ja, c->jupdate == CALIB_JUPDATE_RTR, mode, c->stream));
+        end(pp);
+    }
     void sweep(int mode, const float* J, const float* eta, bool pdl = false) {
         const bool ss = c->formulation == 0 && mode != SWEEP_RESIDUAL;
         ProfPair pp = begin(ss ? (mode == SWEEP_HESSVEC ? 2 : 3) : (mode == SWEEP_HESSVEC ? 1 : 0));
@@ -655,21 +672,23 @@ void enqueue_iteration(Enq& q, bool eval_first, bool gauge) {
     LMArgs la = lm_args(c, ssf ? PARTS_SS_TRIAL : PARTS_DIRECT);       // after the trial sweep
     la_hv.pdl = la.pdl = pdl ? 1 : 0;
     const ConsArgs ca = cons_args(c);
-    if (eval_first) {  // the residual sweep is the direct one in both formulations (it yields g exactly)
-        q.sweep(SWEEP_RESIDUAL, c->J, nullptr);
-        LMArgs l0 = lm_args(c, PARTS_DIRECT);
-        l0.pdl = la.pdl;
-        q.lm_eval(l0, LM_BEGIN_FROM_PARTIALS);
+    LMArgs l0 = lm_args(c, PARTS_DIRECT);
+    l0.pdl = la.pdl;
+    const int begin_mode = eval_first ? LM_BEGIN_FROM_PARTIALS : LM_BEGIN_REUSE;
+    // the residual sweep is the direct one in both formulations (it yields g exactly)
+    if (eval_first) q.sweep(SWEEP_RESIDUAL, c->J, nullptr);
+    if (c->one_launch) {
+        q.jupdate(l0, begin_mode);
     } else {
-        q.lm_eval(la, LM_BEGIN_REUSE);
-    }
-    for (int l = 0; l < c->n_lm; ++l) {
-        for (int k = 0; k < c->n_cg; ++k) {
-            q.sweep(SWEEP_HESSVEC, c->J, c->p, pdl);
-            q.cg_step(la_hv, k == c->n_cg - 1);  // the last one forms the trial point
+        q.lm_eval(eval_first ? l0 : la, begin_mode);
+        for (int l = 0; l < c->n_lm; ++l) {
+            for (int k = 0; k < c->n_cg; ++k) {
+                q.sweep(SWEEP_HESSVEC, c->J, c->p, pdl);
+                q.cg_step(la_hv, k == c->n_cg - 1);  // the last one forms the trial point
+            }
+            q.sweep(SWEEP_TRIAL, c->J, c->x, pdl);
+            q.lm_eval(la, LM_ACCEPT);
         }
-        q.sweep(SWEEP_TRIAL, c->J, c->x, pdl);
-        q.lm_eval(la, LM_ACCEPT);
     }
     ProfPair pp = q.begin(7);
     if (gauge) q.ok(launch_gauge(ca, c->stream));
@@ -938,6 +957,9 @@ int calib_init(calib_ctx** out, int n_stations, int n_baselines, const int32_t* 
 
     auto bail = [&](int rc) { calib_destroy(c); return rc; };
     if (cudaGetDevice(&c->dev) != cudaSuccess) return bail(fail(CALIB_ECUDA, "no CUDA device"));
+    if (cudaDeviceGetAttribute(&c->sms, cudaDevAttrMultiProcessorCount, c->dev) != cudaSuccess || c->sms < 1)
+        return bail(fail(CALIB_ECUDA, "cannot read the SM count"));
+    c->one_launch = c->formulation == 0 && c->jupdate != CALIB_JUPDATE_SAGE && jupdate_plan(N, K, A, c->sms, c->jup);
     if (opt.cuda_stream) {
         c->stream = static_cast<cudaStream_t>(opt.cuda_stream);
     } else {
@@ -949,6 +971,7 @@ int calib_init(calib_ctx** out, int n_stations, int n_baselines, const int32_t* 
     if (pe == cudaSuccess) pe = prepare_lm_kernels();
     if (pe == cudaSuccess) pe = prepare_data_kernels();
     if (pe == cudaSuccess) pe = prepare_ss_kernels();
+    if (pe == cudaSuccess) pe = prepare_jupdate_kernels();
     if (pe != cudaSuccess) return bail(fail(CALIB_ECUDA, std::string("kernel set-up: ") + cudaGetErrorString(pe)));
 
     const size_t vec = (size_t)A * K * N * 8;
@@ -1008,8 +1031,6 @@ int calib_init(calib_ctx** out, int n_stations, int n_baselines, const int32_t* 
     cudaMemset(c->status, 0, sizeof(int));
     cudaMemset(c->st, 0, (size_t)A * sizeof(AgentState));
     cudaMemset(c->prim, 0, (size_t)A * K * sizeof(double));
-    if (cudaDeviceGetAttribute(&c->sms, cudaDevAttrMultiProcessorCount, c->dev) != cudaSuccess || c->sms < 1)
-        return bail(fail(CALIB_ECUDA, "cannot read the SM count"));
     int rc = build_layout(c, nullptr);
     if (rc) return bail(rc);
     rc = set_partition(c, c->part_hv, c->part_hv.m);
@@ -1278,7 +1299,7 @@ int calib_admm_iter(calib_ctx* c, int n_iters, calib_stats* hist) {
         c->launches += 1;
         c->ss_dirty = false;
     }
-    if (c->tune_pending) {
+    if (c->tune_pending && !c->one_launch) {  // the one-launch J-update has no split
         rc = autotune(c);
         if (rc) return rc;
         CK(cudaMemsetAsync(c->status, 0, sizeof(int), c->stream));
@@ -1533,7 +1554,7 @@ int calib_profile_read(calib_ctx* c, int cap, const char** names, double* total_
     if (!c) return fail(CALIB_EINVAL, "ctx is NULL");
     static const char* kNames[calib_ctx::PROF_KINDS] = {"sweep_residual", "sweep_hessvec", "stats_hessvec",
                                                           "stats_trial", "pcg_step", "lm_eval", "stats_pass",
-                                                          "consensus"};
+                                                          "consensus", "jupdate"};
     for (int i = 0; i < calib_ctx::PROF_KINDS && i < cap; ++i) {
         if (names) names[i] = kNames[i];
         if (total_ms) total_ms[i] = c->prof_ms[i];
