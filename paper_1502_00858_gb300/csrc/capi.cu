@@ -148,6 +148,8 @@ struct calib_ctx {
     double* evG = nullptr;
     void* staging = nullptr;
     size_t staging_bytes = 0;
+    double* pred_sources = nullptr;  // table of a prediction
+    size_t pred_bytes = 0;
     // SAGE: one direction's one-direction problem (statistics and per-agent vectors, K = 1)
     float2 *sgU = nullptr, *sgS = nullptr;
     float *sgJ = nullptr, *sgJt = nullptr, *sgY = nullptr, *sgBZ = nullptr, *sgGradg = nullptr, *sgGrad = nullptr;
@@ -508,6 +510,7 @@ int build_layout(calib_ctx* c, const uint8_t* flags) {
     // statistics of flagged baselines stay zero: the statistics pass never writes their positions
     CK(cudaMemset(c->ssU, 0, (size_t)std::max(1LL, c->int_u) * sizeof(float2)));
     CK(cudaMemset(c->ssS, 0, (size_t)std::max(1LL, c->int_s) * sizeof(float2)));
+    CK(cudaMemset(c->gw, 0, (size_t)A * K * N * ((N + 3) / 4 * 4) * sizeof(float)));
     CK(cudaMemcpy(c->desc, c->desc_h.data(), c->desc_h.size() * sizeof(DiagDesc), cudaMemcpyHostToDevice));
     if (!c->slot_h.empty()) {
         CK(cudaMemcpy(c->slot, c->slot_h.data(), c->slot_h.size() * sizeof(int), cudaMemcpyHostToDevice));
@@ -544,6 +547,32 @@ int stage_in(calib_ctx* c, const void* src, size_t bytes, int ptr_kind, const vo
     char* d = static_cast<char*>(c->staging) + staging_off;
     CK(cudaMemcpyAsync(d, src, bytes, cudaMemcpyHostToDevice, c->stream));
     *dev = d;
+    return CALIB_OK;
+}
+
+// Table of a prediction's sources at every frequency, kept with the context up to PREDICT_TABLE bytes. A larger
+// one, and a new one while the stream is being captured or where there is no room, is left out: k_predict
+// then forms the values itself.
+constexpr size_t PREDICT_TABLE = 64u << 20;
+int predict_workspace(calib_ctx* c, PredictArgs& pa) {
+    const size_t want = (size_t)pa.P * pa.K * pa.S * 4 * sizeof(double);
+    pa.sources = nullptr;
+    if (want > PREDICT_TABLE) return CALIB_OK;
+    if (want > c->pred_bytes) {
+        cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+        CK(cudaStreamIsCapturing(c->stream, &cap));
+        if (cap != cudaStreamCaptureStatusNone) return CALIB_OK;
+        CK(cudaStreamSynchronize(c->stream));
+        cudaFree(c->pred_sources);
+        c->pred_sources = nullptr;
+        c->pred_bytes = 0;
+        if (dalloc(&c->pred_sources, want / sizeof(double)) != cudaSuccess) {
+            cudaGetLastError();
+            return CALIB_OK;
+        }
+        c->pred_bytes = want;
+    }
+    pa.sources = c->pred_sources;
     return CALIB_OK;
 }
 
@@ -1102,8 +1131,11 @@ int calib_set_data(calib_ctx* c, const void* vis, const void* coh, const uint8_t
         ia.dst = c->C;
         ia.is_vis = 0;
         CK(launch_ingest(ia, c->stream));
-        CK(launch_gram_weights(c->C, c->desc, c->slot, c->T_d, c->gw, c->A, c->D, c->K, c->N, c->stream));
-        c->launches += 3;
+        c->launches += 2;
+        if (c->formulation == 1) {  // the statistics pass forms the Jacobi weights with S
+            CK(launch_gram_weights(c->C, c->desc, c->slot, c->T_d, c->gw, c->A, c->D, c->K, c->N, c->stream));
+            c->launches += 1;
+        }
         c->coh_set = true;
     }
     c->data_set = true;
@@ -1154,9 +1186,14 @@ int calib_predict(calib_ctx* c, const double* uvw_m, const double* sky, int n_sr
     pa.S = n_src;
     pa.D = c->D;
     pa.Tmax = Tmax;
+    rc = predict_workspace(c, pa);
+    if (rc) return rc;
     CK(launch_predict(pa, c->stream));
-    CK(launch_gram_weights(c->C, c->desc, c->slot, c->T_d, c->gw, c->A, c->D, c->K, c->N, c->stream));
-    c->launches += 2;
+    c->launches += 1 + (pa.sources ? 1 : 0);
+    if (c->formulation == 1) {
+        CK(launch_gram_weights(c->C, c->desc, c->slot, c->T_d, c->gw, c->A, c->D, c->K, c->N, c->stream));
+        c->launches += 1;
+    }
     c->ss_dirty = true;
     c->coh_set = true;
     c->need_eval = true;
@@ -1285,7 +1322,7 @@ int calib_admm_iter(calib_ctx* c, int n_iters, calib_stats* hist) {
             CK(cudaEventCreate(&p1));
             CK(cudaEventRecord(p0, c->stream));
         }
-        CK(launch_ss_stats(c->V, c->C, c->ssU, c->ssS, c->desc, c->slot, c->T_d, c->A, c->D, c->K, c->N, c->Tmax, c->status, c->stream));
+        CK(launch_ss_stats(c->V, c->C, c->ssU, c->ssS, c->gw, c->desc, c->slot, c->T_d, c->A, c->D, c->K, c->N, c->Tmax, c->status, c->stream));
         if (c->profiling) {
             CK(cudaEventRecord(p1, c->stream));
             CK(cudaEventSynchronize(p1));
@@ -1648,7 +1685,7 @@ int calib_autotune(calib_ctx* c, int* split, int* split_trial, int cap, int* can
     if (!c) return fail(CALIB_EINVAL, "ctx is NULL");
     if (!c->data_set || !c->coh_set) return fail(CALIB_ESTATE, "set visibilities and coherencies first");
     if (c->formulation == 0 && c->ss_dirty) {
-        CK(launch_ss_stats(c->V, c->C, c->ssU, c->ssS, c->desc, c->slot, c->T_d, c->A, c->D, c->K, c->N, c->Tmax, c->status, c->stream));
+        CK(launch_ss_stats(c->V, c->C, c->ssU, c->ssS, c->gw, c->desc, c->slot, c->T_d, c->A, c->D, c->K, c->N, c->Tmax, c->status, c->stream));
         c->launches += 1;
         c->ss_dirty = false;
     }
@@ -1711,7 +1748,7 @@ void calib_destroy(calib_ctx* c) {
                     (void*)c->basis_df, (void*)c->Pinv_df, (void*)c->rinv_df, (void*)c->prim_part, (void*)c->pen_part,
                     (void*)c->rec_part, (void*)c->rec_count, (void*)c->stats, (void*)c->iter_counter,
                     (void*)c->status, (void*)c->part_hv.pn, (void*)c->part_tr.pn, (void*)c->evL, (void*)c->evG, (void*)c->T_d, (void*)c->vis_off_d,
-                    (void*)c->coh_off_d, c->staging, (void*)c->ws_prev, (void*)c->ws_mlp, (void*)c->ws_L,
+                    (void*)c->coh_off_d, c->staging, (void*)c->pred_sources, (void*)c->ws_prev, (void*)c->ws_mlp, (void*)c->ws_L,
                     (void*)c->xf_d, (void*)c->ws_chose, (void*)c->sgU, (void*)c->sgS, (void*)c->sgJ, (void*)c->sgJt,
                     (void*)c->sgY, (void*)c->sgBZ, (void*)c->sgGradg, (void*)c->sgGrad, (void*)c->sgX, (void*)c->sgR,
                     (void*)c->sgP, (void*)c->sgGm, (void*)c->sgSt})

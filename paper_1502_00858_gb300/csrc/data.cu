@@ -7,7 +7,7 @@
 // Prediction (Eq. coh): c_pq = sum_s I_s(f) exp(i phi_pq,s) with phi = -2 pi (f/c)
 // (u_pq l + v_pq m + w_pq (n - 1)) and (u,v,w)_pq = (u,v,w)_p - (u,v,w)_q. The phase splits into
 // station phasors E_ps = exp(-2 pi i turns_ps), turns_ps = (f/c)(u_p l + v_p m + w_p (n-1)), so
-// c_pq = sum_s I_s E_ps conj(E_qs). Turns are formed in float64 and reduced to [-1/2, 1/2]
+// c_pq = sum_s I_s E_ps conj(E_qs). Turns are formed in float64 and reduced to [-1/2, 1/2)
 // before the float32 sincospi, so the phase error does not grow with baseline length.
 #include <math.h>
 
@@ -180,82 +180,200 @@ __global__ void __launch_bounds__(RES_THREADS) k_residual(const ResidualArgs a) 
     }
 }
 
-// One CTA per (sample, agent); source chunks sized to fit the phasor table in shared memory.
-__global__ void __launch_bounds__(256) k_predict(const PredictArgs a, int s_chunk) {
-    extern __shared__ __align__(128) unsigned char smem[];  // one declaration for the file's kernels
-    const int t = blockIdx.x, agent = blockIdx.y;
-    const int Ta = a.T[agent];
-    if (t >= Ta) return;
-    const int iv = agent / a.P, fi = agent - iv * a.P;
-    const double f = a.freqs[fi];
-    const int N = a.N, K = a.K;
-    double* lmn = reinterpret_cast<double*>(smem);                        // [K][s_chunk][3] l, m, n - 1
-    float2* E = reinterpret_cast<float2*>(lmn + (size_t)K * s_chunk * 3);  // [K][s_chunk][N]
-    float* flux = reinterpret_cast<float*>(E + (size_t)K * s_chunk * N);  // [K][s_chunk]
-    const double* uvw = a.uvw + (((size_t)iv * a.Tmax + t) * N) * 3;
-    const DiagDesc* dsc_agent = a.desc + (size_t)agent * a.D;
-
-    for (int s0 = 0; s0 < a.S; s0 += s_chunk) {
-        const int ns = min(s_chunk, a.S - s0);
-        // per source: flux at f and its direction (l, m, n - 1), scaled by f / c
-        const double fc = f / C_LIGHT;
-        for (int i = threadIdx.x; i < K * ns; i += blockDim.x) {
-            const int k = i / ns, s = i - k * ns;
-            const double* src = a.sky + ((size_t)k * a.S + s0 + s) * 4;
-            flux[k * s_chunk + s] = (float)(src[2] * pow(f / a.f0, src[3]));
-            const double l = src[0], m = src[1];
-            const double r2 = l * l + m * m;
-            double* d = lmn + ((size_t)k * s_chunk + s) * 3;
-            d[0] = fc * l;
-            d[1] = fc * m;
-            d[2] = fc * (-r2 / (1.0 + sqrt(1.0 - r2)));  // sqrt(1 - l^2 - m^2) - 1, cancellation-free
-        }
-        __syncthreads();
-        for (int i = threadIdx.x; i < K * ns * N; i += blockDim.x) {
-            const int p = i % N;
-            const int ks = i / N;
-            const int k = ks / ns, s = ks - k * ns;
-            const double* d = lmn + ((size_t)k * s_chunk + s) * 3;
-            const double turns = uvw[p * 3 + 0] * d[0] + uvw[p * 3 + 1] * d[1] + uvw[p * 3 + 2] * d[2];
-            const float fr = (float)(turns - rint(turns));
-            float sn, cs;
-            sincospif(2.0f * fr, &sn, &cs);
-            E[((size_t)k * s_chunk + s) * N + p] = make_float2(cs, -sn);  // exp(-2 pi i turns)
-        }
-        __syncthreads();
-        for (int d = 0; d < a.D; ++d) {
-            const DiagDesc dsc = dsc_agent[d];
-            float2* out = a.C + dsc.coff + (size_t)t * dsc.n_pad * K;
-            for (int it = threadIdx.x; it < dsc.n_pad * K; it += blockDim.x) {
-                const int g = it / K, k = it - g * K;
-                float2 c = make_float2(0.f, 0.f);
-                if (g < dsc.n) {
-                    const int sl = a.slot[dsc.slot_off + g];
-                    const int p = sl & 0xff, q = (sl >> 8) & 0xff;
-                    const float2* Ek = E + (size_t)k * s_chunk * N;
-                    const float* fk = flux + k * s_chunk;
-                    for (int s = 0; s < ns; ++s) {
-                        const float2 ep = Ek[s * N + p], eq = Ek[s * N + q];
-                        // I_s E_p conj(E_q)
-                        const float re = ep.x * eq.x + ep.y * eq.y;
-                        const float im = ep.y * eq.x - ep.x * eq.y;
-                        c.x = fmaf(fk[s], re, c.x);
-                        c.y = fmaf(fk[s], im, c.y);
-                    }
-                }
-                if (s0 == 0) {
-                    out[it] = c;
-                } else {
-                    const float2 o = out[it];
-                    out[it] = make_float2(o.x + c.x, o.y + c.y);
-                }
-            }
-        }
-        __syncthreads();
+// ---- prediction
+//
+// What does not depend on the sample is formed once per call: flux and direction (l, m, n - 1) f / c of every
+// source at every frequency, in float64 (k_predict_sources). A table larger than the context keeps is not
+// built; the values are then formed where they are used.
+__device__ __forceinline__ float predict_flux(const double* src, double f, double f0) { return (float)(src[2] * pow(f / f0, src[3])); }
+__device__ __forceinline__ void predict_direction(const double* src, double fc, double (&d)[3]) {
+    const double l = src[0], m = src[1];
+    const double r2 = l * l + m * m;
+    d[0] = fc * l;
+    d[1] = fc * m;
+    d[2] = fc * (-r2 / (1.0 + sqrt(1.0 - r2)));  // sqrt(1 - l^2 - m^2) - 1, cancellation-free
+}
+__global__ void __launch_bounds__(128) k_predict_sources(const PredictArgs a) {
+    const int KS = a.K * a.S;
+    const long long n = (long long)a.P * KS;
+    for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (long long)gridDim.x * blockDim.x) {
+        const double f = a.freqs[i / KS];
+        const double* src = a.sky + (size_t)(i % KS) * 4;
+        double d[3];
+        predict_direction(src, f / C_LIGHT, d);
+        double* o = a.sources + i * 4;
+        o[0] = d[0];
+        o[1] = d[1];
+        o[2] = d[2];
+        o[3] = (double)predict_flux(src, f, a.f0);
     }
 }
 
-// Jacobi weights of one agent: gw[k][o][p] = gw[k][p][o] = s_bk = sum_t |c_btk|^2 for the baseline
+// turns - rint(turns) in float32. The float64 rate is low on this GPU, so the fraction is cut out of the
+// mantissa with integer instructions (64 fractional bits: the same float32 as by rint) from 2^-11 turns on
+// while it has bits there; the rest by rint, in a call, so that it is not executed beside the usual case.
+__device__ __noinline__ float predict_rint_fraction(double turns) { return (float)(turns - rint(turns)); }
+__device__ __forceinline__ float predict_fraction(double turns) {
+    const long long bits = __double_as_longlong(turns);
+    const int shift = (int)((bits >> 52) & 0x7ff) - 1011;  // |turns| = mantissa 2^(shift - 64)
+    if ((unsigned)shift >= 64u) return predict_rint_fraction(turns);
+    const long long frac = (long long)((((unsigned long long)bits & 0xfffffffffffffull) | 0x10000000000000ull) << shift);
+    return __ll2float_rn(bits < 0 ? -frac : frac) * 5.421010862427522e-20f;  // 2^-64
+}
+
+// One CTA per (sample, agent) and group of directions. The sums c_pq = sum_s I_s E_ps conj(E_qs) are products
+// of a station x source matrix with its conjugate transpose: a thread holds a 4 x 4 tile of station pairs
+// (first station in block bp, second in block bq) of one direction, so that a source costs four 16-byte shared loads for
+// 96 arithmetic instructions (one pair a thread: two 8-byte loads for 6). Phasors of one chunk of sources are formed while the
+// chunk before is summed (two buffers, one barrier a chunk). The sums go through shared memory into the
+// slot layout, so that a slot's directions are written together; long sums are cut into parts there.
+// Measured: 62 stations, 5 directions of 100 sources, 640 (sample, agent)s: 465 us against 760 us with one pair a
+// thread; 20 sources, 3200 (sample, agent)s: 690 against 974 us. What bounds it now is the float64 chain of the
+// turns (37 % of that pipe) beside 6 float32 operations a pair and source (31 % of that pipe).
+constexpr int PRED_THREADS = 736;  // five directions of 62 stations (720 tiles) at a time; 80 registers
+// Tiles of station blocks delta apart: with the lower block first where some pair of theirs is at most N / 2
+// apart (held in station order), with the higher block first where some pair is further apart.
+__host__ __device__ inline int predict_tile_fwd(int N, int delta) { return 2 * (delta == 0 ? 1 : 4 * delta - 3) <= N; }
+__host__ __device__ inline int predict_tile_rev(int N, int delta) { return delta > 0 && 2 * (4 * delta + 3) > N; }  // (delta 0: both orders in one tile)
+__host__ __device__ inline int predict_tiles(int N) {
+    const int nb = (N + 3) / 4;
+    int n = 0;
+    for (int delta = 0; delta < nb; ++delta) n += (nb - delta) * (predict_tile_fwd(N, delta) + predict_tile_rev(N, delta));
+    return n;
+}
+constexpr int PRED_SMEM_MAX = 200 * 1024;
+constexpr int PRED_PHASORS = 56 * 1024;  // bytes of the two phasor buffers
+
+__global__ void __launch_bounds__(PRED_THREADS) k_predict(const PredictArgs a, const int KG, const int chunk, const int part) {
+    extern __shared__ __align__(128) unsigned char smem[];  // one declaration for the file's kernels
+    const int N = a.N, K = a.K, S = a.S, N4 = (N + 3) / 4 * 4, nb = N4 / 4, tiles = predict_tiles(N);
+    const int iv = blockIdx.y / a.P, fi = blockIdx.y - iv * a.P, agent = blockIdx.y, t = blockIdx.x, k0 = blockIdx.z * KG;
+    if (t >= a.T[agent]) return;
+    const int kg = min(KG, K - k0), tid = threadIdx.x, nthr = blockDim.x;
+    const double f = a.freqs[fi], fc = f / C_LIGHT;
+    const double* uvw = a.uvw + (((size_t)iv * a.Tmax + t) * N) * 3;
+    const double* sources = a.sources ? a.sources + (size_t)fi * K * S * 4 : nullptr;
+    const int bufn = KG * chunk * N4;
+    float2* E = reinterpret_cast<float2*>(smem);                             // [2][KG][chunk][N4]
+    float* fx = reinterpret_cast<float*>(smem + (size_t)2 * bufn * 8);       // [2][KG][chunk]
+    float2* cs = reinterpret_cast<float2*>(smem + (size_t)2 * KG * chunk * (N4 * 8 + 4) / 16 * 16 + 16);  // [D * N][KG] sums
+
+    // this thread's tile: direction kk, first and second station blocks bp, bq
+    const int kk = tid / tiles;
+    int bp = 0, bq = 0;
+    for (int w = tid - kk * tiles, delta = 0; delta < nb; ++delta) {
+        const int fwd = predict_tile_fwd(N, delta), rev = predict_tile_rev(N, delta), n = nb - delta;
+        if (w < n * (fwd + rev)) {
+            const bool swap = w >= n * fwd;
+            const int b = swap ? w - n * fwd : w;
+            bp = swap ? b + delta : b;
+            bq = swap ? b : b + delta;
+            break;
+        }
+        w -= n * (fwd + rev);
+    }
+    const bool on = kk < kg;
+    float2 acc[4][4];
+#pragma unroll
+    for (int i = 0; i < 4; ++i)
+#pragma unroll
+        for (int j = 0; j < 4; ++j) acc[i][j] = make_float2(0.f, 0.f);
+
+    // Phasors of the sources s0 .. s0 + ns into buffer b, as two planes of station pairs: station p at float4
+    // plane (p >> 1) & 1, block p >> 2, so that consecutive blocks are consecutive 16-byte words. A thread keeps its station.
+    const int rows = nthr / N4, fp = tid % N4, fr0 = tid / N4;
+    const double u0 = fp < N ? uvw[fp * 3] : 0.0, u1 = fp < N ? uvw[fp * 3 + 1] : 0.0, u2 = fp < N ? uvw[fp * 3 + 2] : 0.0;
+    auto form = [&](int s0, int ns, int b) {
+        float2* Eb = E + (size_t)b * bufn + (fp >> 2) * 2 + (fp & 1) + ((fp >> 1) & 1) * (N4 / 2);
+        if (fr0 >= rows) return;
+        int k = fr0 / ns, s = fr0 - k * ns;
+        while (k < kg) {
+            const int src = (k0 + k) * S + s0 + s;
+            double dir[3], w;
+            if (sources) {
+                const double2 u = *reinterpret_cast<const double2*>(sources + (size_t)src * 4), v = *reinterpret_cast<const double2*>(sources + (size_t)src * 4 + 2);
+                dir[0] = u.x;
+                dir[1] = u.y;
+                dir[2] = v.x;
+                w = v.y;
+            } else {
+                predict_direction(a.sky + (size_t)src * 4, fc, dir);
+                w = fp == 0 ? (double)predict_flux(a.sky + (size_t)src * 4, f, a.f0) : 0.0;
+            }
+            float2 e = make_float2(0.f, 0.f);
+            if (fp < N) {
+                const double turns = u0 * dir[0] + u1 * dir[1] + u2 * dir[2];
+                float sn, c;
+                sincospif(2.0f * predict_fraction(turns), &sn, &c);
+                e = make_float2(c, -sn);  // exp(-2 pi i turns)
+            }
+            Eb[(k * chunk + s) * N4] = e;
+            if (fp == 0) fx[b * KG * chunk + k * chunk + s] = (float)w;
+            for (s += rows; s >= ns; s -= ns) ++k;
+        }
+    };
+    // sources of the chunk from s0 on: a chunk ends where a part of the sum ends
+    auto count = [&](int s0) { return min(min(chunk, S - s0), part - s0 % part); };
+    const bool early = (tid >> 5) & 1;
+    form(0, count(0), 0);
+    __syncthreads();
+    for (int s0 = 0, b = 0, ns = 0; s0 < S; s0 += ns, b ^= 1) {
+        ns = count(s0);
+        // Half of the warps form the next phasors before they sum, the others after: the float64 and
+        // transcendental latency of the one runs beside the FMAs of the other.
+        if (early && s0 + ns < S) form(s0 + ns, count(s0 + ns), b ^ 1);
+        if (on) {
+            const float4* Ek = reinterpret_cast<const float4*>(E + (size_t)b * bufn + (size_t)kk * chunk * N4);
+            const float* fk = fx + b * KG * chunk + kk * chunk;
+#pragma unroll 2
+            for (int s = 0; s < ns; ++s) {
+                const float4* Es = Ek + (size_t)s * (N4 / 2);
+                const float4 p01 = Es[bp], p23 = Es[nb + bp], q01 = Es[bq], q23 = Es[nb + bq];
+                const float w = fk[s];
+                const float2 p[4] = {make_float2(p01.x, p01.y), make_float2(p01.z, p01.w), make_float2(p23.x, p23.y), make_float2(p23.z, p23.w)};
+                const float2 q[4] = {make_float2(q01.x, q01.y), make_float2(q01.z, q01.w), make_float2(q23.x, q23.y), make_float2(q23.z, q23.w)};
+#pragma unroll
+                for (int i = 0; i < 4; ++i)
+#pragma unroll
+                    for (int j = 0; j < 4; ++j) {  // I_s E_p conj(E_q): the product rounded before the sum's FMA
+                        const float re = p[i].x * q[j].x + p[i].y * q[j].y;
+                        const float im = p[i].y * q[j].x - p[i].x * q[j].y;
+                        acc[i][j].x = fmaf(w, re, acc[i][j].x);
+                        acc[i][j].y = fmaf(w, im, acc[i][j].y);
+                    }
+            }
+        }
+        // End of a part: its sums to shared memory, position p of diagonal d (each entry by its own thread).
+        if (on && ((s0 + ns) % part == 0 || s0 + ns == S)) {
+#pragma unroll
+            for (int i = 0; i < 4; ++i)
+#pragma unroll
+                for (int j = 0; j < 4; ++j) {
+                    const int p = bp * 4 + i, q = bq * 4 + j;
+                    const int d = q >= p ? q - p : q - p + N;  // the pair's diagonal with p as its first station
+                    if (p < N && q < N && p != q && (2 * d < N || (2 * d == N && p < q))) {
+                        float2* c = cs + ((size_t)(d - 1) * N + p) * KG + kk;
+                        const float2 v = acc[i][j];
+                        *c = s0 + ns <= part ? v : make_float2(c->x + v.x, c->y + v.y);
+                    }
+                    acc[i][j] = make_float2(0.f, 0.f);
+                }
+        }
+        if (!early && s0 + ns < S) form(s0 + ns, count(s0 + ns), b ^ 1);
+        __syncthreads();
+    }
+    const DiagDesc* dsc_agent = a.desc + (size_t)agent * a.D;
+    for (int d = tid >> 5; d < a.D; d += nthr >> 5) {
+        const DiagDesc dsc = dsc_agent[d];
+        float2* out = a.C + dsc.coff + (size_t)t * dsc.n_pad * K + k0;
+        for (int i = tid & 31; i < dsc.n_pad * kg; i += 32) {
+            const int g = i / kg, k = i - g * kg;
+            out[(size_t)g * K + k] = g < dsc.n ? cs[((size_t)d * N + (a.slot[dsc.slot_off + g] & 0xff)) * KG + k] : make_float2(0.f, 0.f);
+        }
+    }
+}
+
+// Jacobi weights of one agent (the direct form; the statistics pass writes them itself): gw[k][o][p] = gw[k][p][o] = s_bk = sum_t |c_btk|^2 for the baseline
 // b = (p, o), zero for flagged baselines and o = p (fixed for the whole calibration). Each entry is
 // written by the one slot that holds its station pair: no atomics.
 // One CTA per (diagonal, agent); the entries no slot writes (the diagonal p = o, flagged pairs,
@@ -297,7 +415,7 @@ constexpr size_t SS_STATS_STAGED_MAX = 200 * 1024;
 template <int KB, bool STAGED>
 __global__ void __launch_bounds__(512, KB > 8 ? 1 : 2) k_ss_stats(const float2* __restrict__ V, const float2* __restrict__ C,
                                                                    float2* __restrict__ U, float2* __restrict__ S,
-                                                                   const DiagDesc* desc, const int* slot, const int* T,
+                                                                   float* __restrict__ gw, int N, const DiagDesc* desc, const int* slot, const int* T,
                                                                    int D, int K, int NP, int* status) {
     extern __shared__ __align__(128) unsigned char smem[];
     __shared__ __align__(8) uint64_t bar;
@@ -375,6 +493,15 @@ __global__ void __launch_bounds__(512, KB > 8 ? 1 : 2) k_ss_stats(const float2* 
 #pragma unroll
         for (int l = 0; l < KB; ++l)
             if (l >= k && l < K) so[l - k] = srow[l];
+        // S_kk is the Jacobi weight of the baseline (see k_gram_weights), at both of its stations
+        float skk = 0.f;
+#pragma unroll
+        for (int l = 0; l < KB; ++l)
+            if (l == k) skk = srow[l].x;
+        const int sl = slot[dsc.slot_off + g], f = sl & 0xff, sc = (sl >> 8) & 0xff;
+        float* W = gw + ((size_t)agent * K + k) * N * NP;
+        W[(size_t)f * NP + sc] = skk;
+        W[(size_t)sc * NP + f] = skk;
     }
 }
 
@@ -391,7 +518,7 @@ __global__ void k_check_finite(const float* x, long long n, int* status) {
 cudaError_t prepare_data_kernels() {
     const auto attr = cudaFuncAttributeMaxDynamicSharedMemorySize;
     const int st = (int)SS_STATS_STAGED_MAX;
-    cudaError_t e = cudaFuncSetAttribute(k_predict, attr, 100 * 1024);
+    cudaError_t e = cudaFuncSetAttribute(k_predict, attr, PRED_SMEM_MAX);
     if (e == cudaSuccess) e = cudaFuncSetAttribute(k_ss_stats<4, true>, attr, st);
     if (e == cudaSuccess) e = cudaFuncSetAttribute(k_ss_stats<8, true>, attr, st);
     if (e == cudaSuccess) e = cudaFuncSetAttribute(k_ss_stats<MAX_K, true>, attr, st);
@@ -413,14 +540,31 @@ cudaError_t launch_residual(const ResidualArgs& a, cudaStream_t s) {
     k_residual<<<grid, RES_THREADS, (size_t)a.K * 2 * RES_THREADS * sizeof(float4), s>>>(a);
     return cudaGetLastError();
 }
+// Directions and sources at a time: as many directions as have tiles for the threads, sources to fill the
+// phasor buffers; the sums of a group use the same shared memory afterwards.
+size_t predict_smem(int N, int KG, int chunk) {
+    const size_t N4 = (N + 3) / 4 * 4;
+    return (size_t)2 * KG * chunk * (N4 * 8 + 4) / 16 * 16 + 16 + (size_t)(N / 2) * N * KG * 8;
+}
 cudaError_t launch_predict(const PredictArgs& a, cudaStream_t s) {
-    const size_t budget = 96 * 1024;
-    int s_chunk = a.S;
-    // per source: its N station phasors (8 B each), its flux (4 B) and l, m, n - 1 (24 B)
-    while (s_chunk > 1 && (size_t)a.K * s_chunk * (a.N * 8 + 28) > budget) s_chunk = (s_chunk + 1) / 2;
-    const size_t smem = (size_t)a.K * s_chunk * (a.N * 8 + 28);
-    dim3 grid(a.Tmax, a.A);
-    k_predict<<<grid, 256, smem, s>>>(a, s_chunk);
+    const int N4 = (a.N + 3) / 4 * 4, tiles = predict_tiles(a.N);
+    // all tiles of a direction have to have a thread: at most 561 (N = 128)
+    int KG = std::max(1, std::min(a.K, PRED_THREADS / tiles));
+    while (KG > 1 && predict_smem(a.N, KG, 1) > PRED_SMEM_MAX) --KG;
+    const int groups = (a.K + KG - 1) / KG;
+    KG = (a.K + groups - 1) / groups;
+    const int chunk = std::max(1, std::min(a.S, PRED_PHASORS / (2 * KG * (N4 * 8 + 4))));
+    if (a.sources) {
+        const long long n = (long long)a.P * a.K * a.S;
+        k_predict_sources<<<(unsigned)std::min<long long>((n + 127) / 128, 4096), 128, 0, s>>>(a);
+        const cudaError_t e = cudaGetLastError();
+        if (e != cudaSuccess) return e;
+    }
+    const int threads = std::max(64, (KG * tiles + 31) / 32 * 32);
+    // sources summed in one chain (float32 round-off grows with its length); the parts are added in order
+    int part = a.S;
+    while (part > 1 && (size_t)a.K * part * (a.N * 8 + 28) > 96 * 1024) part = (part + 1) / 2;
+    k_predict<<<dim3(a.Tmax, a.A, groups), threads, predict_smem(a.N, KG, chunk), s>>>(a, KG, chunk, part);
     return cudaGetLastError();
 }
 cudaError_t launch_gram_weights(const float2* C, const DiagDesc* desc, const int* slot, const int* T, float* gw,
@@ -434,25 +578,25 @@ cudaError_t launch_gram_weights(const float2* C, const DiagDesc* desc, const int
 size_t ss_stats_smem(int N, int K, int Tmax) { return (size_t)Tmax * ((N + 3) / 4 * 4) * (32 + 8 * K); }
 
 template <int KB>
-cudaError_t ss_stats_go(const float2* V, const float2* C, float2* U, float2* S, const DiagDesc* desc, const int* slot,
+cudaError_t ss_stats_go(const float2* V, const float2* C, float2* U, float2* S, float* gw, int N, const DiagDesc* desc, const int* slot,
                         const int* T, int A, int D, int K, int NP, size_t smem, int* status, cudaStream_t s) {
     const int threads = std::min(512, ((NP * K + 31) / 32) * 32);
     dim3 grid(D, A);
     if (smem <= SS_STATS_STAGED_MAX)
-        k_ss_stats<KB, true><<<grid, threads, smem, s>>>(V, C, U, S, desc, slot, T, D, K, NP, status);
+        k_ss_stats<KB, true><<<grid, threads, smem, s>>>(V, C, U, S, gw, N, desc, slot, T, D, K, NP, status);
     else
-        k_ss_stats<KB, false><<<grid, threads, 0, s>>>(V, C, U, S, desc, slot, T, D, K, NP, status);
+        k_ss_stats<KB, false><<<grid, threads, 0, s>>>(V, C, U, S, gw, N, desc, slot, T, D, K, NP, status);
     return cudaGetLastError();
 }
 
-cudaError_t launch_ss_stats(const float2* V, const float2* C, float2* U, float2* S, const DiagDesc* desc,
+cudaError_t launch_ss_stats(const float2* V, const float2* C, float2* U, float2* S, float* gw, const DiagDesc* desc,
                             const int* slot, const int* T, int A, int D, int K, int N, int Tmax, int* status,
                             cudaStream_t s) {
     const int NP = (N + 3) / 4 * 4;
     const size_t smem = ss_stats_smem(N, K, Tmax);
-    if (K <= 4) return ss_stats_go<4>(V, C, U, S, desc, slot, T, A, D, K, NP, smem, status, s);
-    if (K <= 8) return ss_stats_go<8>(V, C, U, S, desc, slot, T, A, D, K, NP, smem, status, s);
-    return ss_stats_go<MAX_K>(V, C, U, S, desc, slot, T, A, D, K, NP, smem, status, s);
+    if (K <= 4) return ss_stats_go<4>(V, C, U, S, gw, N, desc, slot, T, A, D, K, NP, smem, status, s);
+    if (K <= 8) return ss_stats_go<8>(V, C, U, S, gw, N, desc, slot, T, A, D, K, NP, smem, status, s);
+    return ss_stats_go<MAX_K>(V, C, U, S, gw, N, desc, slot, T, A, D, K, NP, smem, status, s);
 }
 
 cudaError_t launch_check_finite(const float* x, long long n, int* status, cudaStream_t s) {
