@@ -268,7 +268,7 @@ __device__ void project_out_gauge(const Blk (&j)[BPT], Blk (&g)[BPT], int K, int
 }
 
 // Jacobi blocks G_pk = sum_o s_(p,o)k J_ok^H J_ok at the CTA's J (held by the threads), from the
-// dense weights gw (thread (k, p) reads its 16-byte aligned row, all loads independent) and the
+// dense weights gw (all loads independent) and the
 // products J_ok^H J_ok staged in sm (KN*4 floats).
 template <int BPT>
 __device__ void gram_blocks(const LMArgs& a, int agent, const Blk (&j)[BPT], float* sm, float (&G)[BPT][4]) {
@@ -292,24 +292,19 @@ __device__ void gram_blocks(const LMArgs& a, int agent, const Blk (&j)[BPT], flo
         G[i][0] = G[i][1] = G[i][2] = G[i][3] = 0.f;
         if (blk >= KN) continue;
         const int k = blk / N, p = blk - k * N;
-        const int NW4 = (N + 3) / 4;
-        const float4* W = reinterpret_cast<const float4*>(a.gw + (((size_t)agent * K + k) * N + p) * NW4 * 4);
+        // the weights are symmetric: read along a row, consecutive threads read consecutive words
+        const int NW = (N + 3) / 4 * 4;
+        const float* W = a.gw + ((size_t)agent * K + k) * N * NW + p;
         const float4* X = reinterpret_cast<const float4*>(sm) + k * N;
         float g0 = 0.f, g1 = 0.f, g2 = 0.f, g3 = 0.f;
 #pragma unroll 16
-        for (int o4 = 0; o4 < NW4; ++o4) {
-            const float4 w4 = __ldg(W + o4);
-            const float wv[4] = {w4.x, w4.y, w4.z, w4.w};
-#pragma unroll
-            for (int q = 0; q < 4; ++q) {
-                const int o = 4 * o4 + q;
-                if (o >= N) break;  // row padding
-                const float4 x = X[o];
-                g0 = fmaf(wv[q], x.x, g0);
-                g1 = fmaf(wv[q], x.y, g1);
-                g2 = fmaf(wv[q], x.z, g2);
-                g3 = fmaf(wv[q], x.w, g3);
-            }
+        for (int o = 0; o < N; ++o) {
+            const float w = __ldg(W + (size_t)o * NW);
+            const float4 x = X[o];
+            g0 = fmaf(w, x.x, g0);
+            g1 = fmaf(w, x.y, g1);
+            g2 = fmaf(w, x.z, g2);
+            g3 = fmaf(w, x.w, g3);
         }
         G[i][0] = g0; G[i][1] = g1; G[i][2] = g2; G[i][3] = g3;
         reinterpret_cast<float4*>(a.Gm + (size_t)agent * KN * 4)[blk] = make_float4(g0, g1, g2, g3);

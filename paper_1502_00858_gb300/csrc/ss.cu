@@ -7,7 +7,8 @@
 //   trial pass:    W_k = sum_t conj(c_tk) R_t = U_k - sum_l S_kl P_l (P_l = J_pl J_ql^H) at J, and at
 //                  J' = J + x: W'_k = W_k - sum_l S_kl dP_l with the exact model change
 //                  dP_l = x_pl J_ql^H + J_pl x_ql^H + x_pl x_ql^H; the data-cost decrease is
-//                  g(J) - g(J') = sum_k Re <dP_k, 2 W_k - (S dP)_k> (Frobenius inner product).
+//                  g(J) - g(J') = sum_k Re <dP_k, 2 W_k - (S dP)_k> (Frobenius inner product), or, from K = 4 on,
+//                  W'_k = U_k - sum_l S_kl P'_l at once and sum_k Re <dP_k, 2 W'_k> + sum_kl Re(S_kl <dP_k, dP_l>).
 // The identities are exact; the per-pass work and traffic no longer depend on the number of samples.
 //
 // Work split: the A*D (agent, circulant diagonal) items are cut into gridDim.x equal contiguous
@@ -47,6 +48,8 @@ __global__ void __launch_bounds__(SMALL ? 128 : 256,
     constexpr int NST = nst<HV>();
     constexpr float sg = HV ? 1.f : -1.f;  // station terms: + in the Hessian pass, - (gradient) in the trial pass
     constexpr bool UG = ss_u_global(HV, KB);  // the trial pass reads U from global memory (not staged)
+    // Trial pass: W' formed at J' at once, the decrease as Re <dP, 2 W' + S dP> with the last term as a Hermitian form.
+    constexpr bool QF = !HV && KB >= SS_FORM_KMIN;
     extern __shared__ __align__(128) unsigned char smem[];
     const int N = a.N, D = a.D, NP = a.NP;
     const int K = EXACT ? KB : a.K;
@@ -192,11 +195,14 @@ __global__ void __launch_bounds__(SMALL ? 128 : 256,
 #pragma unroll
         for (int k = 0; k < KB; ++k) Xd[k] = Xo[k] = make_float2(0.f, 0.f);
         if (active) {
-            float2 Yd[HV ? 1 : KB], Yo[HV ? 1 : KB];    // trial: row rr of (S dP)_k
+            float2 Yd[HV || QF ? 1 : KB], Yo[HV || QF ? 1 : KB];  // trial: row rr of (S dP)_k
             float2 dPd[HV ? 1 : KB], dPo[HV ? 1 : KB];  // trial: row rr of dP_l
             if (!HV) {
 #pragma unroll
-                for (int k = 0; k < KB; ++k) Yd[k] = Yo[k] = dPd[k] = dPo[k] = make_float2(0.f, 0.f);
+                for (int k = 0; k < KB; ++k) {
+                    dPd[k] = dPo[k] = make_float2(0.f, 0.f);
+                    if (!QF) Yd[QF ? 0 : k] = Yo[QF ? 0 : k] = make_float2(0.f, 0.f);
+                }
             }
 #pragma unroll
             for (int l = 0; l < KB; ++l) {
@@ -212,8 +218,8 @@ __global__ void __launch_bounds__(SMALL ? 128 : 256,
                     qo = cdot2_acc(cdot2_acc(z2, Ef[l], jso), Jf[l], eso);
                 } else {   // P_l = J_f J_s^H;  dP_l = J'_f J'_s^H - P_l = x_f J'_s^H + J_f x_s^H, x = J' - J
                     const float4 xf = f4sub(Ef[l], Jf[l]);
-                    qd = cdot2_acc(z2, Jf[l], jsd);
-                    qo = cdot2_acc(z2, Jf[l], jso);
+                    qd = QF ? cdot2_acc(z2, Ef[l], esd) : cdot2_acc(z2, Jf[l], jsd);
+                    qo = QF ? cdot2_acc(z2, Ef[l], eso) : cdot2_acc(z2, Jf[l], jso);
                     pd = cdot2_acc(cdot2_acc(z2, xf, esd), Jf[l], f4sub(esd, jsd));
                     po = cdot2_acc(cdot2_acc(z2, xf, eso), Jf[l], f4sub(eso, jso));
                     dPd[l] = pd;
@@ -228,9 +234,9 @@ __global__ void __launch_bounds__(SMALL ? 128 : 256,
                     if (k > l) skl.y = -skl.y;
                     cmac(Xd[k], skl, qd);
                     cmac(Xo[k], skl, qo);
-                    if (!HV) {
-                        cmac(Yd[k], skl, pd);
-                        cmac(Yo[k], skl, po);
+                    if (!HV && !QF) {
+                        cmac(Yd[QF ? 0 : k], skl, pd);
+                        cmac(Yo[QF ? 0 : k], skl, po);
                     }
                 }
             }
@@ -241,13 +247,45 @@ __global__ void __launch_bounds__(SMALL ? 128 : 256,
                     if (k >= K) continue;
                     const float2* u = Us + (((size_t)g * K + k) * 2 + rr) * 2;
                     const float2 ud = UG ? __ldg(u + rr) : u[rr], uo = UG ? __ldg(u + ro) : u[ro];
-                    const float2 Wd = f2sub(ud, Xd[k]);  // W_k at J
+                    const float2 Wd = f2sub(ud, Xd[k]);  // W_k at J (QF: at J')
                     const float2 Wo = f2sub(uo, Xo[k]);
+                    if constexpr (QF) {
+                        dcf = fmaf(dPd[k].x, Wd.x, fmaf(dPd[k].y, Wd.y, dcf));
+                        dcf = fmaf(dPo[k].x, Wo.x, fmaf(dPo[k].y, Wo.y, dcf));
+                        Xd[k] = Wd;
+                        Xo[k] = Wo;
+                        continue;
+                    }
                     // decrease: Re[conj(dP_k) (2 W_k - (S dP)_k)], this row
-                    dcf = fmaf(dPd[k].x, 2.f * Wd.x - Yd[k].x, fmaf(dPd[k].y, 2.f * Wd.y - Yd[k].y, dcf));
-                    dcf = fmaf(dPo[k].x, 2.f * Wo.x - Yo[k].x, fmaf(dPo[k].y, 2.f * Wo.y - Yo[k].y, dcf));
-                    Xd[k] = f2sub(Wd, Yd[k]);  // W'_k at J' = J + x
-                    Xo[k] = f2sub(Wo, Yo[k]);
+                    const float2 yd = Yd[QF ? 0 : k], yo = Yo[QF ? 0 : k];
+                    dcf = fmaf(dPd[k].x, 2.f * Wd.x - yd.x, fmaf(dPd[k].y, 2.f * Wd.y - yd.y, dcf));
+                    dcf = fmaf(dPo[k].x, 2.f * Wo.x - yo.x, fmaf(dPo[k].y, 2.f * Wo.y - yo.y, dcf));
+                    Xd[k] = f2sub(Wd, yd);  // W'_k at J' = J + x
+                    Xo[k] = f2sub(Wo, yo);
+                }
+                if constexpr (QF) {  // 2 Re <dP, W'> + sum_kl Re(conj(dP_k) S_kl dP_l), this row
+                    float own_k = 0.f, cross = 0.f;
+#pragma unroll
+                    for (int k = 0; k < KB; ++k) {
+                        if (k >= K) continue;
+                        const float2* Sk = Ss + k * K - k * (k - 1) / 2;  // entry (k, l) at l - k
+                        const float n2 = fmaf(dPd[k].x, dPd[k].x, fmaf(dPd[k].y, dPd[k].y, fmaf(dPo[k].x, dPo[k].x, dPo[k].y * dPo[k].y)));
+                        own_k = fmaf(Sk[0].x, n2, own_k);
+#pragma unroll
+                        for (int l = k + 1; l < KB; ++l) {
+                            if (l >= K) continue;
+                            float re = dPd[k].x * dPd[l].x, im = dPd[k].x * dPd[l].y;
+                            re = fmaf(dPd[k].y, dPd[l].y, re);
+                            im = fmaf(-dPd[k].y, dPd[l].x, im);
+                            re = fmaf(dPo[k].x, dPo[l].x, re);
+                            im = fmaf(dPo[k].x, dPo[l].y, im);
+                            re = fmaf(dPo[k].y, dPo[l].y, re);
+                            im = fmaf(-dPo[k].y, dPo[l].x, im);
+                            const float2 skl = Sk[l - k];
+                            cross = fmaf(skl.x, re, fmaf(-skl.y, im, cross));
+                        }
+                    }
+                    dcf = 2.f * (dcf + cross) + own_k;
                 }
                 dcost += (double)dcf;
             }

@@ -12,6 +12,11 @@ namespace ss {
 // measured no faster for the Hessian pass).
 template <bool HV> __host__ __device__ constexpr int nst() { return 2; }
 constexpr int BAR_BYTES = 64;  // barrier area, keeps what follows 16-byte aligned
+// From this bucket on the trial pass forms <dP, S dP> as a Hermitian form (10 FMAs a row and direction pair)
+// instead of (S dP)_k for every k (16 FMAs, and the registers of K more blocks): 1018 to 703 us at K = 10 (1024 agents
+// of 62 stations; 216 to 0 spilled bytes), 70 to 64 us at K = 5 (320 agents). Below, the pass is no shorter
+// by it, and few directions hold the gauge so weakly that its results should not move.
+constexpr int SS_FORM_KMIN = 4;
 constexpr int HV1_KMAX = 5;    // largest K of the one-thread-per-slot Hessian kernel (register budget)
 
 
