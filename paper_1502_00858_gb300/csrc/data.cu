@@ -230,6 +230,7 @@ __device__ __forceinline__ float predict_fraction(double turns) {
 // Measured: 62 stations, 5 directions of 100 sources, 640 (sample, agent)s: 465 us against 760 us with one pair a
 // thread; 20 sources, 3200 (sample, agent)s: 690 against 974 us. What bounds it now is the float64 chain of the
 // turns (37 % of that pipe) beside 6 float32 operations a pair and source (31 % of that pipe).
+constexpr int PRED_THREADS_SMALL = 288;
 constexpr int PRED_THREADS = 736;  // five directions of 62 stations (720 tiles) at a time; 80 registers
 // Tiles of station blocks delta apart: with the lower block first where some pair of theirs is at most N / 2
 // apart (held in station order), with the higher block first where some pair is further apart.
@@ -244,7 +245,8 @@ __host__ __device__ inline int predict_tiles(int N) {
 constexpr int PRED_SMEM_MAX = 200 * 1024;
 constexpr int PRED_PHASORS = 56 * 1024;  // bytes of the two phasor buffers
 
-__global__ void __launch_bounds__(PRED_THREADS) k_predict(const PredictArgs a, const int KG, const int chunk, const int part) {
+template <int MAXT, int MINB>
+__global__ void __launch_bounds__(MAXT, MINB) k_predict(const PredictArgs a, const int KG, const int chunk, const int part) {
     extern __shared__ __align__(128) unsigned char smem[];  // one declaration for the file's kernels
     const int N = a.N, K = a.K, S = a.S, N4 = (N + 3) / 4 * 4, nb = N4 / 4, tiles = predict_tiles(N);
     const int iv = blockIdx.y / a.P, fi = blockIdx.y - iv * a.P, agent = blockIdx.y, t = blockIdx.x, k0 = blockIdx.z * KG;
@@ -518,7 +520,8 @@ __global__ void k_check_finite(const float* x, long long n, int* status) {
 cudaError_t prepare_data_kernels() {
     const auto attr = cudaFuncAttributeMaxDynamicSharedMemorySize;
     const int st = (int)SS_STATS_STAGED_MAX;
-    cudaError_t e = cudaFuncSetAttribute(k_predict, attr, PRED_SMEM_MAX);
+    cudaError_t e = cudaFuncSetAttribute(k_predict<PRED_THREADS, 1>, attr, PRED_SMEM_MAX);
+    if (e == cudaSuccess) e = cudaFuncSetAttribute(k_predict<PRED_THREADS_SMALL, 3>, attr, PRED_SMEM_MAX);
     if (e == cudaSuccess) e = cudaFuncSetAttribute(k_ss_stats<4, true>, attr, st);
     if (e == cudaSuccess) e = cudaFuncSetAttribute(k_ss_stats<8, true>, attr, st);
     if (e == cudaSuccess) e = cudaFuncSetAttribute(k_ss_stats<MAX_K, true>, attr, st);
@@ -549,11 +552,12 @@ size_t predict_smem(int N, int KG, int chunk) {
 cudaError_t launch_predict(const PredictArgs& a, cudaStream_t s) {
     const int N4 = (a.N + 3) / 4 * 4, tiles = predict_tiles(a.N);
     // all tiles of a direction have to have a thread: at most 561 (N = 128)
-    int KG = std::max(1, std::min(a.K, PRED_THREADS / tiles));
+    const bool small = tiles <= PRED_THREADS_SMALL;
+    int KG = std::max(1, std::min(a.K, (small ? PRED_THREADS_SMALL : PRED_THREADS) / tiles));
     while (KG > 1 && predict_smem(a.N, KG, 1) > PRED_SMEM_MAX) --KG;
     const int groups = (a.K + KG - 1) / KG;
     KG = (a.K + groups - 1) / groups;
-    const int chunk = std::max(1, std::min(a.S, PRED_PHASORS / (2 * KG * (N4 * 8 + 4))));
+    const int chunk = std::max(1, std::min(a.S, (small ? PRED_PHASORS / 2 : PRED_PHASORS) / (2 * KG * (N4 * 8 + 4))));
     if (a.sources) {
         const long long n = (long long)a.P * a.K * a.S;
         k_predict_sources<<<(unsigned)std::min<long long>((n + 127) / 128, 4096), 128, 0, s>>>(a);
@@ -564,7 +568,12 @@ cudaError_t launch_predict(const PredictArgs& a, cudaStream_t s) {
     // sources summed in one chain (float32 round-off grows with its length); the parts are added in order
     int part = a.S;
     while (part > 1 && (size_t)a.K * part * (a.N * 8 + 28) > 96 * 1024) part = (part + 1) / 2;
-    k_predict<<<dim3(a.Tmax, a.A, groups), threads, predict_smem(a.N, KG, chunk), s>>>(a, KG, chunk, part);
+    const dim3 grid(a.Tmax, a.A, groups);
+    const size_t smem = predict_smem(a.N, KG, chunk);
+    if (small)
+        k_predict<PRED_THREADS_SMALL, 3><<<grid, threads, smem, s>>>(a, KG, chunk, part);
+    else
+        k_predict<PRED_THREADS, 1><<<grid, threads, smem, s>>>(a, KG, chunk, part);
     return cudaGetLastError();
 }
 cudaError_t launch_gram_weights(const float2* C, const DiagDesc* desc, const int* slot, const int* T, float* gw,
