@@ -224,12 +224,16 @@ cudaError_t launch_identity(float* J, long long n_blocks, cudaStream_t s);
 struct IngestArgs {
     const float2* src;          // user layout [A][B][T_a][w] (w = 4 for V, K for C)
     const long long* src_off;   // [A] float2 offset of each agent's [B][T_a][w] block
-    const uint8_t* flags;       // unused here (slots already compacted)
+    const int2* flagged;        // (agent, baseline) of the baselines that have no slot
+    int* status;
     float2* dst;
     const DiagDesc* desc; const int* slot; const int* slot_b; const int* T;
-    int A, D, K, is_vis;
+    int A, D, K, is_vis, n_flagged, slots_max;
 };
+// Moves the data into the internal layout and checks all of them (status bit STATUS_NONFINITE).
 cudaError_t launch_ingest(const IngestArgs& a, cudaStream_t s);
+// Zeroes the flagged baselines of a user-layout array [A][B][T_a][w].
+cudaError_t launch_zero_flagged(const int2* flagged, int n, const long long* off, const int* T, int w, float2* out, cudaStream_t s);
 cudaError_t launch_extract_coh(const IngestArgs& a, float2* user_dst, cudaStream_t s);
 struct ResidualArgs {
     const float2* V; const float2* C;  // internal layouts
@@ -255,7 +259,6 @@ struct PredictArgs {
 cudaError_t launch_predict(const PredictArgs& a, cudaStream_t s);
 cudaError_t launch_gram_weights(const float2* C, const DiagDesc* desc, const int* slot, const int* T, float* gw,
                                 int A, int D, int K, int N, cudaStream_t s);
-cudaError_t launch_check_finite(const float* x, long long n, int* status, cudaStream_t s);
 // Statistics into the full circulant layout and the Jacobi weights (positions of flagged baselines are not written).
 cudaError_t launch_ss_stats(const float2* V, const float2* C, float2* U, float2* S, float* gw, const DiagDesc* desc,
                             const int* slot, const int* T, int A, int D, int K, int N, int Tmax, int* status,

@@ -122,7 +122,8 @@ struct calib_ctx {
     bool ss_dirty = true;
     DiagDesc* desc = nullptr;
     int *slot = nullptr, *slot_b = nullptr, *T_d = nullptr;
-    int2* inc = nullptr;
+    int2* flagged = nullptr;  // (agent, baseline) of the flagged baselines
+    int n_flagged = 0;
     float* gw = nullptr;  // [A][K][N][N] Jacobi weights
     long long *vis_off_d = nullptr, *coh_off_d = nullptr;
     float *J = nullptr, *Jt = nullptr, *Y = nullptr, *BZ = nullptr, *gradg = nullptr, *grad = nullptr;
@@ -401,6 +402,8 @@ void free_layout(calib_ctx* c) {
     cudaFree(c->desc); c->desc = nullptr;
     cudaFree(c->slot); c->slot = nullptr;
     cudaFree(c->slot_b); c->slot_b = nullptr;
+    cudaFree(c->flagged); c->flagged = nullptr;
+    c->n_flagged = 0;
     cudaFree(c->gw); c->gw = nullptr;
     cudaFree(c->ssU); c->ssU = nullptr;
     cudaFree(c->ssS); c->ssS = nullptr;
@@ -504,6 +507,12 @@ int build_layout(calib_ctx* c, const uint8_t* flags) {
     CK(dalloc(&c->desc, c->desc_h.size()));
     CK(dalloc(&c->slot, c->slot_h.size()));
     CK(dalloc(&c->slot_b, c->slot_b_h.size()));
+    std::vector<int2> flagged;
+    for (long long i = 0; flags && i < (long long)A * c->B; ++i)
+        if (flags[i]) flagged.push_back(make_int2((int)(i / c->B), (int)(i % c->B)));
+    CK(dalloc(&c->flagged, flagged.size()));
+    if (!flagged.empty()) CK(cudaMemcpy(c->flagged, flagged.data(), flagged.size() * sizeof(int2), cudaMemcpyHostToDevice));
+    c->n_flagged = (int)flagged.size();
     CK(dalloc(&c->gw, (size_t)A * K * N * ((N + 3) / 4 * 4)));
     CK(dalloc(&c->ssU, (size_t)c->int_u));
     CK(dalloc(&c->ssS, (size_t)c->int_s));
@@ -1109,29 +1118,31 @@ int calib_set_data(calib_ctx* c, const void* vis, const void* coh, const uint8_t
     ia.A = c->A;
     ia.D = c->D;
     ia.K = c->K;
+    ia.flagged = c->flagged;
+    ia.n_flagged = c->n_flagged;
+    ia.slots_max = c->slots_max;
+    ia.status = c->status;
     const void* dv = nullptr;
     int rc = stage_in(c, vis, (size_t)c->user_v * sizeof(float2), ptr_kind, &dv);
     if (rc) return rc;
     CK(cudaMemsetAsync(c->status, 0, sizeof(int), c->stream));
-    CK(launch_check_finite(static_cast<const float*>(dv), c->user_v * 2, c->status, c->stream));
     ia.src = static_cast<const float2*>(dv);
     ia.src_off = c->vis_off_d;
     ia.dst = c->V;
     ia.is_vis = 1;
     CK(launch_ingest(ia, c->stream));
-    c->launches += 2;
+    c->launches += 1 + (c->n_flagged ? 1 : 0);
     c->ss_dirty = true;
     if (coh) {
         const void* dc = nullptr;
         rc = stage_in(c, coh, (size_t)c->user_c * sizeof(float2), ptr_kind, &dc);
         if (rc) return rc;
-        CK(launch_check_finite(static_cast<const float*>(dc), c->user_c * 2, c->status, c->stream));
         ia.src = static_cast<const float2*>(dc);
         ia.src_off = c->coh_off_d;
         ia.dst = c->C;
         ia.is_vis = 0;
         CK(launch_ingest(ia, c->stream));
-        c->launches += 2;
+        c->launches += 1 + (c->n_flagged ? 1 : 0);
         if (c->formulation == 1) {  // the statistics pass forms the Jacobi weights with S
             CK(launch_gram_weights(c->C, c->desc, c->slot, c->T_d, c->gw, c->A, c->D, c->K, c->N, c->stream));
             c->launches += 1;
@@ -1212,7 +1223,7 @@ int calib_get_coherencies(calib_ctx* c, void* coh, int ptr_kind) {
         if (rc) return rc;
         dst = c->staging;
     }
-    CK(cudaMemsetAsync(dst, 0, bytes, c->stream));
+    CK(launch_zero_flagged(c->flagged, c->n_flagged, c->coh_off_d, c->T_d, c->K, static_cast<float2*>(dst), c->stream));
     IngestArgs ia{};
     ia.desc = c->desc;
     ia.slot = c->slot;
@@ -1223,8 +1234,9 @@ int calib_get_coherencies(calib_ctx* c, void* coh, int ptr_kind) {
     ia.K = c->K;
     ia.src_off = c->coh_off_d;
     ia.dst = c->C;
+    ia.slots_max = c->slots_max;
     CK(launch_extract_coh(ia, static_cast<float2*>(dst), c->stream));
-    c->launches += 1;
+    c->launches += 1 + (c->n_flagged ? 1 : 0);
     if (ptr_kind == 0) {
         CK(cudaMemcpyAsync(coh, dst, bytes, cudaMemcpyDeviceToHost, c->stream));
         CK(cudaStreamSynchronize(c->stream));
@@ -1247,9 +1259,8 @@ int calib_residual(calib_ctx* c, const int32_t* subtract, int correct_dir, void*
         if (rc) return rc;
         dst = c->staging;
     }
-    // flagged baselines have no slot in the layout: zero them (every output when any is flagged)
-    if (std::any_of(c->flags_h.begin(), c->flags_h.end(), [](uint8_t f) { return f != 0; }))
-        CK(cudaMemsetAsync(dst, 0, bytes, c->stream));
+    // flagged baselines have no slot in the layout
+    CK(launch_zero_flagged(c->flagged, c->n_flagged, c->vis_off_d, c->T_d, 4, static_cast<float2*>(dst), c->stream));
     ResidualArgs ra{};
     ra.V = c->V;
     ra.C = c->C;
@@ -1267,7 +1278,7 @@ int calib_residual(calib_ctx* c, const int32_t* subtract, int correct_dir, void*
     ra.mask = mask;
     ra.correct = correct_dir;
     CK(launch_residual(ra, c->stream));
-    c->launches += 1;
+    c->launches += 1 + (c->n_flagged ? 1 : 0);
     if (ptr_kind == 0) {
         CK(cudaMemcpyAsync(out, dst, bytes, cudaMemcpyDeviceToHost, c->stream));
         CK(cudaStreamSynchronize(c->stream));
