@@ -591,6 +591,21 @@ int copy_out(calib_ctx* c, void* dst, const void* dev_src, size_t bytes, int ptr
     return CALIB_OK;
 }
 
+// Whether kernels with 16-byte accesses can use a caller's array directly.
+bool usable_in_place(const void* p, int ptr_kind) { return p && ptr_kind == 1 && (reinterpret_cast<uintptr_t>(p) & 15) == 0; }
+bool overlap(const void* p, size_t np, const void* q, size_t nq) {
+    const uintptr_t a = reinterpret_cast<uintptr_t>(p), b = reinterpret_cast<uintptr_t>(q);
+    return p && q && a < b + nq && b < a + np;
+}
+// A caller's input where it is, or copied to own.
+int in_place(calib_ctx* c, const void* src, float* own, size_t bytes, int ptr_kind, const float** p) {
+    *p = static_cast<const float*>(src);
+    if (usable_in_place(src, ptr_kind)) return CALIB_OK;
+    CK(cudaMemcpyAsync(own, src, bytes, ptr_kind == 1 ? cudaMemcpyDeviceToDevice : cudaMemcpyHostToDevice, c->stream));
+    *p = own;
+    return CALIB_OK;
+}
+
 int check_status(calib_ctx* c) {
     int st = 0;
     CK(cudaMemcpy(&st, c->status, sizeof(int), cudaMemcpyDeviceToHost));
@@ -1540,17 +1555,25 @@ int calib_eval(calib_ctx* c, const void* Jin, double* L, double* g, void* grad, 
     if (!valid_kind(ptr_kind)) return fail(CALIB_EINVAL, "ptr_kind must be 0 (host) or 1 (device)");
     if (!c->data_set || !c->coh_set) return fail(CALIB_ESTATE, "set visibilities and coherencies first");
     const size_t vb = (size_t)c->A * c->K * c->N * 8 * sizeof(float);
-    CK(cudaMemcpyAsync(c->evJ, Jin, vb, ptr_kind == 1 ? cudaMemcpyDeviceToDevice : cudaMemcpyHostToDevice, c->stream));
+    // device arrays that the kernels' 16-byte accesses can take are used where they are, others (and host
+    // arrays) through the context's own; grad may be J itself: each of its blocks is read before it is written
+    const float* J = nullptr;
+    int rc = in_place(c, Jin, c->evJ, vb, ptr_kind, &J);
+    if (rc) return rc;
+    const size_t ab = (size_t)c->A * sizeof(double);
+    const bool apart = !overlap(L, ab, Jin, vb) && !overlap(g, ab, Jin, vb) && !overlap(L, ab, grad, vb) && !overlap(g, ab, grad, vb) &&
+                       !overlap(L, ab, g, ab) && (grad == Jin || !overlap(grad, vb, Jin, vb));
+    const bool here = ptr_kind == 1 && apart, grad_here = here && usable_in_place(grad, ptr_kind);
     CK(cudaMemsetAsync(c->status, 0, sizeof(int), c->stream));
-    CK(launch_sweep(sweep_args(c, SWEEP_RESIDUAL, c->evJ, nullptr), SWEEP_RESIDUAL, c->stream));
+    CK(launch_sweep(sweep_args(c, SWEEP_RESIDUAL, J, nullptr), SWEEP_RESIDUAL, c->stream));
     LMArgs la = lm_args(c, PARTS_DIRECT);
-    la.Jt = c->evJ;
-    CK(launch_eval_output(la, c->evOut, c->evL, c->evG, c->stream));
+    la.Jt = const_cast<float*>(J);
+    CK(launch_eval_output(la, grad_here ? static_cast<float*>(grad) : c->evOut, here && L ? L : c->evL, here && g ? g : c->evG,
+                          c->stream));
     c->launches += 2;
-    int rc;
-    if (grad && (rc = copy_out(c, grad, c->evOut, vb, ptr_kind))) return rc;
-    if (L && (rc = copy_out(c, L, c->evL, (size_t)c->A * sizeof(double), ptr_kind))) return rc;
-    if (g && (rc = copy_out(c, g, c->evG, (size_t)c->A * sizeof(double), ptr_kind))) return rc;
+    if (grad && !grad_here && (rc = copy_out(c, grad, c->evOut, vb, ptr_kind))) return rc;
+    if (L && !here && (rc = copy_out(c, L, c->evL, ab, ptr_kind))) return rc;
+    if (g && !here && (rc = copy_out(c, g, c->evG, ab, ptr_kind))) return rc;
     if (ptr_kind == 0) {
         CK(cudaStreamSynchronize(c->stream));
         return check_status(c);
@@ -1563,17 +1586,18 @@ int calib_hessvec(calib_ctx* c, const void* Jin, const void* eta, void* out, int
     if (!valid_kind(ptr_kind)) return fail(CALIB_EINVAL, "ptr_kind must be 0 (host) or 1 (device)");
     if (!c->coh_set) return fail(CALIB_ESTATE, "set coherencies first");
     const size_t vb = (size_t)c->A * c->K * c->N * 8 * sizeof(float);
-    const cudaMemcpyKind kind = ptr_kind == 1 ? cudaMemcpyDeviceToDevice : cudaMemcpyHostToDevice;
-    CK(cudaMemcpyAsync(c->evJ, Jin, vb, kind, c->stream));
-    CK(cudaMemcpyAsync(c->evE, eta, vb, kind, c->stream));
-    CK(cudaMemsetAsync(c->status, 0, sizeof(int), c->stream));
-    CK(launch_sweep(sweep_args(c, SWEEP_HESSVEC, c->evJ, c->evE), SWEEP_HESSVEC, c->stream));
-    LMArgs la = lm_args(c, PARTS_DIRECT);
-    la.p = c->evE;
-    CK(launch_hv_output(la, c->evOut, c->stream));
-    c->launches += 2;
-    int rc = copy_out(c, out, c->evOut, vb, ptr_kind);
+    const float *J = nullptr, *E = nullptr;  // as in calib_eval; out may be J or eta
+    int rc = in_place(c, Jin, c->evJ, vb, ptr_kind, &J);
+    if (rc == CALIB_OK) rc = in_place(c, eta, c->evE, vb, ptr_kind, &E);
     if (rc) return rc;
+    const bool out_here = usable_in_place(out, ptr_kind) && (out == eta || !overlap(out, vb, eta, vb));
+    CK(cudaMemsetAsync(c->status, 0, sizeof(int), c->stream));
+    CK(launch_sweep(sweep_args(c, SWEEP_HESSVEC, J, E), SWEEP_HESSVEC, c->stream));
+    LMArgs la = lm_args(c, PARTS_DIRECT);
+    la.p = const_cast<float*>(E);
+    CK(launch_hv_output(la, out_here ? static_cast<float*>(out) : c->evOut, c->stream));
+    c->launches += 2;
+    if (!out_here && (rc = copy_out(c, out, c->evOut, vb, ptr_kind))) return rc;
     if (ptr_kind == 0) {
         CK(cudaStreamSynchronize(c->stream));
         return check_status(c);

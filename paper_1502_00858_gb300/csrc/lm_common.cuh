@@ -62,17 +62,6 @@ __device__ __forceinline__ float block_max(float v, float* red) {
     for (int k = 1; k < nw; ++k) m = fmaxf(m, red[k]);
     return m;
 }
-// float64 variant for the values returned to the caller (calib_eval).
-__device__ double block_sum_d(double v, double* red) {
-    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5, nw = blockDim.x >> 5;
-    for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-    if (lane == 0) red[w] = v;
-    __syncthreads();
-    double s = 0.0;
-    for (int k = 0; k < nw; ++k) s += red[k];
-    return s;
-}
-
 // (G + lam I)^-1 of a Hermitian G (g00, g11, re g01, im g01), in the same form.
 __device__ __forceinline__ float4 precond_inverse(const float (&G)[4], float lam) {
     const float a = G[0] + lam, c = G[1] + lam, br = G[2], bi = G[3];

@@ -18,7 +18,7 @@
 // first element of at most one slot and the second of at most one, so the station sums are
 // accumulated in shared memory in two barrier-separated phases without atomics: the order of
 // every addition is fixed, and the result is bitwise reproducible.
-// Data tiles (all slots of one diagonal, TT samples) are streamed from HBM into a 3-stage
+// Data tiles (all slots of one diagonal, TT samples) are streamed from HBM into a 2-stage
 // shared-memory ring with cp.async.bulk (TMA bulk copies) completing on mbarriers; every wait
 // is bounded and reports a timeout through the status word instead of hanging.
 #include "calib_internal.cuh"
@@ -27,7 +27,9 @@
 namespace calib {
 namespace {
 
-constexpr int NST = 3;
+// Two stages of up to 24 KB and one barrier each: three CTAs an SM at 62 stations, K = 5. Residual pass there (320
+// agents of 10 samples, 436 MB): 132 us; with three stages (two CTAs an SM) 157, with two barriers a stage 165.
+constexpr int NST = 2;
 
 
 __device__ __forceinline__ float2 f2add(float2 a, float2 b) { return make_float2(a.x + b.x, a.y + b.y); }
@@ -67,18 +69,19 @@ __global__ void __launch_bounds__(512) k_sweep(const SweepArgs a, const int stag
 
     unsigned char* stage = smem;
     uint64_t* bar = reinterpret_cast<uint64_t*>(smem + NST * stage_bytes);
-    float2* Js = reinterpret_cast<float2*>(bar + NST);  // [K][N][4]
+    float2* Js = reinterpret_cast<float2*>(bar + NST);  // [K][N][4], 16-byte aligned
     float2* Es = Js + KN4;                                // [K][N][4] direction (Hessian) / step x (trial)
     float2* acc = (HV || TR) ? (Es + KN4) : Es;           // [K][N][4] station sums
     double* red = reinterpret_cast<double*>(acc + KN4);   // [64]
 
-    const float2* Jg = reinterpret_cast<const float2*>(a.J) + (size_t)agent * KN4;
-    for (int i = tid; i < KN4; i += nthr) Js[i] = Jg[i];
-    if (HV || TR) {
-        const float2* Eg = reinterpret_cast<const float2*>(a.eta) + (size_t)agent * KN4;
-        for (int i = tid; i < KN4; i += nthr) Es[i] = Eg[i];
+    const float4* Jg = reinterpret_cast<const float4*>(a.J) + (size_t)agent * KN4 / 2;
+    const float4* Eg = reinterpret_cast<const float4*>(a.eta) + (size_t)agent * KN4 / 2;
+#pragma unroll 4
+    for (int i = tid; i < KN4 / 2; i += nthr) {
+        reinterpret_cast<float4*>(Js)[i] = __ldg(Jg + i);
+        if (HV || TR) reinterpret_cast<float4*>(Es)[i] = __ldg(Eg + i);
+        reinterpret_cast<float4*>(acc)[i] = make_float4(0.f, 0.f, 0.f, 0.f);
     }
-    for (int i = tid; i < KN4; i += nthr) acc[i] = make_float2(0.f, 0.f);
 
     const int Ta = a.T[agent];
     const int d0 = 1 + chunk * a.chunk_diags;
@@ -154,19 +157,20 @@ __global__ void __launch_bounds__(512) k_sweep(const SweepArgs a, const int stag
                 }
             }
         }
-        __syncthreads();  // every thread is done with the buffer that stage s + NST - 1 reuses
-        if (tid == 0 && s + NST - 1 < S) {
-            fence_proxy_async_smem();
-            issue(s + NST - 1);
-        }
         const bool ok = mbar_wait_bounded(&bar[s % NST], (uint32_t)((s / NST) & 1));
         if (__syncthreads_or(!ok)) {
             if (tid == 0) {
                 atomicOr(a.status, STATUS_TIMEOUT);
-                const int last = min(S - 1, s + NST - 1);
+                const int last = min(S - 1, s + NST - 2);  // issued so far
                 for (int s2 = s; s2 <= last; ++s2) mbar_wait_bounded(&bar[s2 % NST], (uint32_t)((s2 / NST) & 1));
             }
             return;
+        }
+        // The one barrier of a stage: it has landed for every thread, and every thread is done with the stage
+        // before, whose buffer the next copy takes.
+        if (tid == 0 && s + NST - 1 < S) {
+            fence_proxy_async_smem();
+            issue(s + NST - 1);
         }
 
         const int t0 = tile * a.TT, nt = min(a.TT, Ta - t0);
@@ -265,8 +269,8 @@ __global__ void __launch_bounds__(512) k_sweep(const SweepArgs a, const int stag
     }
     __syncthreads();
 
-    float2* out = reinterpret_cast<float2*>(a.part) + ((size_t)agent * a.n_chunks + chunk) * KN4;
-    for (int i = tid; i < KN4; i += nthr) out[i] = acc[i];
+    float4* out = reinterpret_cast<float4*>(a.part) + ((size_t)agent * a.n_chunks + chunk) * KN4 / 2;
+    for (int i = tid; i < KN4 / 2; i += nthr) out[i] = reinterpret_cast<const float4*>(acc)[i];
     if (!HV) {
         for (int o = 16; o > 0; o >>= 1) {
             cost += __shfl_down_sync(0xffffffffu, cost, o);
