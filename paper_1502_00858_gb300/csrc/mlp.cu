@@ -62,11 +62,13 @@ template <> struct IsBf16<__nv_bfloat16> { static constexpr bool value = true; }
 constexpr int GT_M = 64, GT_N = 64, GT_K = 16, GT_LD = GT_K + 4;
 constexpr int SPLITK_MAX = 16;  // K-splits of a weight-gradient product
 
-template <typename TAE, typename TBE, bool TA, bool TB, int EPI>
+// SUMS: the CTAs of the first column tile also write the sums of op(A)'s rows over their k (the bias gradient
+// beside a weight gradient) to row_sums + blockIdx.z * M.
+template <typename TAE, typename TBE, bool TA, bool TB, int EPI, bool SUMS>
 __global__ void __launch_bounds__(128) k_gemm(int M, int N, int K, const TAE* __restrict__ A, int lda,
                                               const TBE* __restrict__ B, int ldb, float* __restrict__ C, int ldc,
                                               const __nv_bfloat16* __restrict__ bias, const float* __restrict__ mask,
-                                              int ldm, int k_chunk) {
+                                              int ldm, int k_chunk, float* __restrict__ row_sums) {
     constexpr bool A_EXACT = IsBf16<TAE>::value, B_EXACT = IsBf16<TBE>::value;
     constexpr int PER = GT_M * GT_K / 128;  // tile elements a thread stages per operand
     __shared__ float As[GT_M][GT_LD];  // As[m][k]
@@ -119,11 +121,16 @@ __global__ void __launch_bounds__(128) k_gemm(int M, int N, int K, const TAE* __
             Bs[nn][kq] = rb[q];
         }
     };
+    float rsum = 0.f;  // row tid & 63, half of the k of every tile
     if (kb < ke) fetch(kb);
     for (int k0 = kb; k0 < ke; k0 += GT_K) {
         stage();
         __syncthreads();
         if (k0 + GT_K < ke) fetch(k0 + GT_K);
+        if (SUMS && blockIdx.x == 0) {
+#pragma unroll
+            for (int q = 0; q < GT_K / 2; ++q) rsum += As[threadIdx.x & 63][(threadIdx.x >> 6) * (GT_K / 2) + q];
+        }
 #pragma unroll
         for (int ks = 0; ks < GT_K; ks += 8) {
             uint32_t ah[2][4], al[2][4], bh[4][2], bl[4][2];
@@ -183,14 +190,10 @@ __global__ void __launch_bounds__(128) k_gemm(int M, int N, int K, const TAE* __
                 if (EPI == EPI_MASK) v = mask[(size_t)m * ldm + n] > 0.f ? v : 0.f;
                 Cz[(size_t)m * ldc + n] = v;
             }
-}
-
-// C = sum of the split-K partials in split order (a fixed order: results do not depend on timing).
-__global__ void k_sum_splits(const float* part, int splits, long long n, float* C) {
-    for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (long long)gridDim.x * blockDim.x) {
-        float s = part[i];
-        for (int z = 1; z < splits; ++z) s += part[(size_t)z * n + i];
-        C[i] = s;
+    if (SUMS && blockIdx.x == 0) {
+        if (threadIdx.x >= 64) As[threadIdx.x & 63][0] = rsum;
+        __syncthreads();
+        if (threadIdx.x < 64 && m0 + (int)threadIdx.x < M) row_sums[(size_t)blockIdx.z * M + m0 + threadIdx.x] = rsum + As[threadIdx.x][0];
     }
 }
 
@@ -199,27 +202,17 @@ template <typename TAE, typename TBE, bool TA, bool TB, int EPI>
 cudaError_t gemm(int M, int N, int K, const TAE* A, int lda, const TBE* B, int ldb, float* C, int ldc,
                  const __nv_bfloat16* bias, const float* mask, int ldm, cudaStream_t s) {
     dim3 grid((N + GT_N - 1) / GT_N, (M + GT_M - 1) / GT_M, 1);
-    k_gemm<TAE, TBE, TA, TB, EPI><<<grid, 128, 0, s>>>(M, N, K, A, lda, B, ldb, C, ldc, bias, mask, ldm,
-                                                        (K + GT_K - 1) / GT_K * GT_K);
+    k_gemm<TAE, TBE, TA, TB, EPI, false><<<grid, 128, 0, s>>>(M, N, K, A, lda, B, ldb, C, ldc, bias, mask, ldm,
+                                                              (K + GT_K - 1) / GT_K * GT_K, nullptr);
     return cudaGetLastError();
 }
 
-// Split-K for a product with few output tiles and a long K (the weight gradients, K = rows): up to
-// `splits` CTAs per tile, each over a 16-aligned share of K, their partials summed by k_sum_splits.
-// work: splits * M * N floats; C is a dense M x N array.
-template <typename TAE, typename TBE, bool TA, bool TB>
-cudaError_t gemm_splitk(int M, int N, int K, const TAE* A, int lda, const TBE* B, int ldb, float* C, float* work,
-                        int splits, cudaStream_t s) {
-    const int chunk = ((K + splits - 1) / splits + GT_K - 1) / GT_K * GT_K;
-    splits = chunk > 0 ? (K + chunk - 1) / chunk : 1;
-    if (splits <= 1) return gemm<TAE, TBE, TA, TB, EPI_STORE>(M, N, K, A, lda, B, ldb, C, N, nullptr, nullptr, 0, s);
-    dim3 grid((N + GT_N - 1) / GT_N, (M + GT_M - 1) / GT_M, splits);
-    k_gemm<TAE, TBE, TA, TB, EPI_STORE><<<grid, 128, 0, s>>>(M, N, K, A, lda, B, ldb, work, N, nullptr, nullptr, 0, chunk);
-    cudaError_t e = cudaGetLastError();
-    if (e != cudaSuccess) return e;
-    const long long n = (long long)M * N;
-    k_sum_splits<<<(unsigned)std::min<long long>((n + 255) / 256, 1024), 256, 0, s>>>(work, splits, n, C);
-    return cudaGetLastError();
+// Weight gradient of one layer, g^T h (out x in, summed over the rows): few output tiles over a long K, so up
+// to `splits` CTAs per tile, each over a 16-aligned share of the rows; partials [splits][out][in] to part and
+// the bias gradient's [splits][out] to sums, added up by k_finish in split order. Returns the splits used.
+int grad_splits(int rows, int splits, int* chunk) {
+    *chunk = ((rows + splits - 1) / splits + GT_K - 1) / GT_K * GT_K;
+    return std::max(1, (rows + *chunk - 1) / *chunk);
 }
 
 // dY = 2 (x[:, :8] + y - target) / n and per-block partial sums of the squared error.
@@ -243,43 +236,48 @@ __global__ void k_mse(const float* X, int n_in, const float* Y, const float* T, 
     if (threadIdx.x == 0) part[blockIdx.x] = red[0];
 }
 
-__global__ void k_sum_parts(const double* part, int np, int n, double* out) {
-    if (threadIdx.x == 0 && blockIdx.x == 0) {
+// What a gradient's last kernel needs of each layer.
+constexpr int MAX_LAYERS = 17;
+struct LayerGrads {
+    long long off_w[MAX_LAYERS], off_b[MAX_LAYERS], part[MAX_LAYERS], sums[MAX_LAYERS];  // parameters; partials in the workspace
+    int size_w[MAX_LAYERS], size_b[MAX_LAYERS], splits[MAX_LAYERS], n;
+};
+
+// Gradient of every parameter from the split partials (in split order: results do not depend on timing), the
+// loss from the blocks' shares, and with ADAM the AdamW step (decoupled decay) on the float32 master weights
+// with fresh bfloat16 copies. One launch for all layers: 13 launches a training step instead of 25, whose latency
+// is what a step of a small network costs.
+template <bool ADAM>
+__global__ void __launch_bounds__(256) k_finish(const LayerGrads L, const float* work, float* grad, long long np, const double* loss_part,
+                                                int n_loss, int rows, double* loss, float* w, __nv_bfloat16* wb, float* m, float* v,
+                                                float lr, float b1, float b2, float c1, float c2, float eps, float wd) {
+    if (blockIdx.x == 0 && threadIdx.x < 32) {
         double s = 0.0;
-        for (int i = 0; i < np; ++i) s += part[i];
-        *out = s / n;
+        for (int i = threadIdx.x; i < n_loss; i += 32) s += loss_part[i];
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+        if (threadIdx.x == 0) *loss = s / rows;
     }
-}
-
-// db[c] = sum_r g[r][c]: 32 columns per block, 8 row groups, fixed-order combination.
-__global__ void k_colsum(const float* g, int n, int cols, float* db) {
-    __shared__ float red[8][33];
-    const int c = blockIdx.x * 32 + (threadIdx.x & 31), grp = threadIdx.x >> 5;
-    float s = 0.f;
-    if (c < cols)
-        for (int r = grp; r < n; r += 8) s += g[(size_t)r * cols + c];
-    red[grp][threadIdx.x & 31] = s;
-    __syncthreads();
-    if (grp == 0 && c < cols) {
-        float t = 0.f;
-        for (int i = 0; i < 8; ++i) t += red[i][threadIdx.x & 31];
-        db[c] = t;
-    }
-}
-
-// AdamW (decoupled decay) on the float32 master weights; refresh the bfloat16 copies.
-__global__ void k_adamw(float* w, __nv_bfloat16* wb, float* m, float* v, const float* g, long long np, float lr,
-                        float b1, float b2, float c1, float c2, float eps, float wd) {
     for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < np; i += (long long)gridDim.x * blockDim.x) {
-        const float gi = g[i];
-        const float mi = b1 * m[i] + (1.f - b1) * gi;
-        const float vi = b2 * v[i] + (1.f - b2) * gi * gi;
-        m[i] = mi;
-        v[i] = vi;
-        const float upd = (mi / c1) / (sqrtf(vi / c2) + eps) + wd * w[i];
-        const float wi = w[i] - lr * upd;
-        w[i] = wi;
-        wb[i] = __float2bfloat16_rn(wi);
+        int l = 0;
+        while (l + 1 < L.n && i >= L.off_w[l + 1]) ++l;
+        const bool bias = i >= L.off_b[l];
+        const float* p = work + (bias ? L.sums[l] + (i - L.off_b[l]) : L.part[l] + (i - L.off_w[l]));
+        const int size = bias ? L.size_b[l] : L.size_w[l];
+        float gi = p[0];
+#pragma unroll 4
+        for (int z = 1; z < L.splits[l]; ++z) gi += p[(size_t)z * size];
+        grad[i] = gi;
+        if (ADAM) {
+            const float mi = b1 * m[i] + (1.f - b1) * gi;
+            const float vi = b2 * v[i] + (1.f - b2) * gi * gi;
+            m[i] = mi;
+            v[i] = vi;
+            const float upd = (mi / c1) / (sqrtf(vi / c2) + eps) + wd * w[i];
+            const float wi = w[i] - lr * upd;
+            w[i] = wi;
+            wb[i] = __float2bfloat16_rn(wi);
+        }
     }
 }
 
@@ -338,7 +336,10 @@ struct MlpNet {
     int cap = 0;
     std::vector<float*> act;
     float *X = nullptr, *T = nullptr, *g1 = nullptr, *g2 = nullptr, *pred = nullptr;
-    float* splitk = nullptr;  // split-K partials of the weight gradients: SPLITK_MAX x the largest layer
+    float* splitk = nullptr;  // split-K partials of the weight and bias gradients of every layer
+    calib::LayerGrads lay{};
+    int max_splits[calib::MAX_LAYERS] = {};  // about two CTAs per SM
+    int loss_parts = 0;
     int sms = 1;              // SM count of the device
     double *part = nullptr, *loss = nullptr;
     cudaStream_t stream = nullptr;
@@ -389,25 +390,24 @@ cudaError_t forward(MlpNet* n, const float* X, int rows) {
     return e;
 }
 
-// Gradient of the mean squared error of x[:, :8] + y against T into n->grad; loss into n->loss.
+// Gradient of the mean squared error of x[:, :8] + y against T, as partials that finish() adds up.
 cudaError_t backward(MlpNet* n, const float* X, const float* T, int rows) {
     const int L = (int)n->out_dim.size();
     const unsigned nb = grid_for((long long)rows * n->n_out);
     k_mse<<<nb, 256, 0, n->stream>>>(X, n->n_in, n->act[L - 1], T, n->g1, rows, n->n_out, n->part);
-    k_sum_parts<<<1, 32, 0, n->stream>>>(n->part, (int)nb, rows, n->loss);
+    n->loss_parts = (int)nb;
     cudaError_t e = cudaGetLastError();
     float* g = n->g1;
     float* other = n->g2;
     for (int l = L - 1; l >= 0 && e == cudaSuccess; --l) {
         const float* h_in = l == 0 ? X : n->act[l - 1];
         const int in = n->in_dim[l], out = n->out_dim[l];
-        // dW = g^T h_in  (out x in): few output tiles over a long K (the rows), so split K
-        const int tiles = ((out + GT_M - 1) / GT_M) * ((in + GT_N - 1) / GT_N);
-        const int splits = std::max(1, std::min(SPLITK_MAX, 2 * n->sms / tiles));  // about two CTAs per SM
-        e = gemm_splitk<float, float, true, false>(out, in, rows, g, out, h_in, in, n->grad + n->off_w[l], n->splitk,
-                                                   splits, n->stream);
-        if (e != cudaSuccess) break;
-        k_colsum<<<(out + 31) / 32, 256, 0, n->stream>>>(g, rows, out, n->grad + n->off_b[l]);
+        int chunk;
+        const int splits = grad_splits(rows, n->max_splits[l], &chunk);
+        n->lay.splits[l] = splits;
+        const dim3 grid((in + GT_N - 1) / GT_N, (out + GT_M - 1) / GT_M, splits);
+        k_gemm<float, float, true, false, EPI_STORE, true><<<grid, 128, 0, n->stream>>>(
+            out, in, rows, g, out, h_in, in, n->splitk + n->lay.part[l], in, nullptr, nullptr, 0, chunk, n->splitk + n->lay.sums[l]);
         e = cudaGetLastError();
         if (l > 0 && e == cudaSuccess) {
             // g_prev = (g W) masked by the ReLU of the layer below
@@ -417,6 +417,21 @@ cudaError_t backward(MlpNet* n, const float* X, const float* T, int rows) {
         }
     }
     return e;
+}
+
+// The gradient into n->grad, the loss into n->loss, and with adam the optimiser step.
+cudaError_t finish(MlpNet* n, int rows, bool adam, float lr, float wd) {
+    const unsigned nb = grid_for(n->n_params);
+    const float b1 = 0.9f, b2 = 0.999f;
+    if (adam) {
+        const float c1 = 1.f - (float)std::pow((double)b1, (double)n->t), c2 = 1.f - (float)std::pow((double)b2, (double)n->t);
+        k_finish<true><<<nb, 256, 0, n->stream>>>(n->lay, n->splitk, n->grad, n->n_params, n->part, n->loss_parts, rows, n->loss, n->master, n->wb,
+                                                  n->m, n->v, lr, b1, b2, c1, c2, 1e-8f, wd);
+    } else {
+        k_finish<false><<<nb, 256, 0, n->stream>>>(n->lay, n->splitk, n->grad, n->n_params, n->part, n->loss_parts, rows, n->loss, nullptr, nullptr,
+                                                   nullptr, nullptr, 0.f, b1, b2, 1.f, 1.f, 0.f, 0.f);
+    }
+    return cudaGetLastError();
 }
 
 }  // namespace
@@ -478,12 +493,25 @@ int calib_mlp_create(calib_mlp** out, int n_in, int width, int depth, int n_out,
     if (e == cudaSuccess) e = cudaMalloc(&n->v, off * sizeof(float));
     if (e == cudaSuccess) e = cudaMalloc(&n->grad, off * sizeof(float));
     if (e == cudaSuccess) e = cudaMalloc(&n->part, 4096 * sizeof(double));
-    long long largest = 0;
-    for (size_t l = 0; l < n->in_dim.size(); ++l) largest = std::max(largest, (long long)n->in_dim[l] * n->out_dim[l]);
-    if (e == cudaSuccess) e = cudaMalloc(&n->splitk, (size_t)calib::SPLITK_MAX * largest * sizeof(float));
     int dev = 0;
     if (e == cudaSuccess) e = cudaGetDevice(&dev);
     if (e == cudaSuccess) e = cudaDeviceGetAttribute(&n->sms, cudaDevAttrMultiProcessorCount, dev);
+    long long work = 0;
+    n->lay.n = (int)n->in_dim.size();
+    for (int l = 0; l < n->lay.n; ++l) {
+        const int in = n->in_dim[l], out = n->out_dim[l];
+        const int tiles = ((out + calib::GT_M - 1) / calib::GT_M) * ((in + calib::GT_N - 1) / calib::GT_N);
+        n->max_splits[l] = std::max(1, std::min(calib::SPLITK_MAX, 2 * n->sms / tiles));
+        n->lay.off_w[l] = n->off_w[l];
+        n->lay.off_b[l] = n->off_b[l];
+        n->lay.size_w[l] = in * out;
+        n->lay.size_b[l] = out;
+        n->lay.part[l] = work;
+        work += (long long)n->max_splits[l] * in * out;
+        n->lay.sums[l] = work;
+        work += (long long)n->max_splits[l] * out;
+    }
+    if (e == cudaSuccess) e = cudaMalloc(&n->splitk, (size_t)work * sizeof(float));
     if (e == cudaSuccess) e = cudaMalloc(&n->loss, sizeof(double));
     if (e == cudaSuccess) e = cudaMemset(n->master, 0, off * sizeof(float));
     if (e == cudaSuccess) e = cudaMemset(n->wb, 0, off * sizeof(__nv_bfloat16));
@@ -538,9 +566,11 @@ int calib_mlp_forward(calib_mlp* h, const float* X, float* Y, int rows, int ptr_
     return CALIB_OK;
 }
 
-int calib_mlp_grad(calib_mlp* h, const float* X, const float* T, int rows, float* grad, double* loss, int ptr_kind) {
-    if (!h || !X || !T || rows < 1) return mfail(CALIB_EINVAL, "mlp, X, T and rows >= 1 are required");
-    MlpNet* n = &h->net;
+}  // extern "C"
+
+namespace {
+// Forward and backward pass of a batch: the gradient's partials.
+int mlp_passes(MlpNet* n, const float* X, const float* T, int rows, int ptr_kind) {
     MCK(calib::ensure_cap(n, rows));
     const float *Xd = X, *Td = T;
     if (ptr_kind == 0) {
@@ -551,6 +581,18 @@ int calib_mlp_grad(calib_mlp* h, const float* X, const float* T, int rows, float
     }
     MCK(calib::forward(n, Xd, rows));
     MCK(calib::backward(n, Xd, Td, rows));
+    return CALIB_OK;
+}
+}  // namespace
+
+extern "C" {
+
+int calib_mlp_grad(calib_mlp* h, const float* X, const float* T, int rows, float* grad, double* loss, int ptr_kind) {
+    if (!h || !X || !T || rows < 1) return mfail(CALIB_EINVAL, "mlp, X, T and rows >= 1 are required");
+    MlpNet* n = &h->net;
+    const int rc = mlp_passes(n, X, T, rows, ptr_kind);
+    if (rc) return rc;
+    MCK(calib::finish(n, rows, false, 0.f, 0.f));
     const cudaMemcpyKind k = ptr_kind == 1 ? cudaMemcpyDeviceToDevice : cudaMemcpyDeviceToHost;
     if (grad) MCK(cudaMemcpyAsync(grad, n->grad, n->n_params * sizeof(float), k, n->stream));
     if (loss) MCK(cudaMemcpyAsync(loss, n->loss, sizeof(double), k, n->stream));
@@ -561,20 +603,16 @@ int calib_mlp_grad(calib_mlp* h, const float* X, const float* T, int rows, float
 int calib_mlp_train_step(calib_mlp* h, const float* X, const float* T, int rows, float lr, float weight_decay,
                          double* loss, int ptr_kind) {
     if (!h) return mfail(CALIB_EINVAL, "mlp is NULL");
+    if (!X || !T || rows < 1) return mfail(CALIB_EINVAL, "mlp, X, T and rows >= 1 are required");
     MlpNet* n = &h->net;
-    int rc = calib_mlp_grad(h, X, T, rows, nullptr, nullptr, ptr_kind);
+    const int rc = mlp_passes(n, X, T, rows, ptr_kind);
     if (rc) return rc;
     n->t += 1;
-    const float b1 = 0.9f, b2 = 0.999f;
-    const float c1 = 1.f - (float)std::pow((double)b1, (double)n->t), c2 = 1.f - (float)std::pow((double)b2, (double)n->t);
-    calib::k_adamw<<<calib::grid_for(n->n_params), 256, 0, n->stream>>>(n->master, n->wb, n->m, n->v, n->grad, n->n_params,
-                                                                         lr, b1, b2, c1, c2, 1e-8f, weight_decay);
-    MCK(cudaGetLastError());
-    if (loss) {
+    MCK(calib::finish(n, rows, true, lr, weight_decay));
+    if (loss)
         MCK(cudaMemcpyAsync(loss, n->loss, sizeof(double), ptr_kind == 1 ? cudaMemcpyDeviceToDevice : cudaMemcpyDeviceToHost,
                             n->stream));
-        if (ptr_kind == 0) MCK(cudaStreamSynchronize(n->stream));
-    }
+    if (ptr_kind == 0) MCK(cudaStreamSynchronize(n->stream));  // the host rows are read, the loss is there
     return CALIB_OK;
 }
 
