@@ -837,12 +837,20 @@ int autotune(calib_ctx* c) {
         LMArgs la_tr = lm_args(c, ssf ? PARTS_SS_TRIAL : PARTS_DIRECT);
         la_hv.timing = 1;
         la_tr.Jt = c->J;
+        // Launched as the iteration's graph does (programmatic dependent launch: how well a split's CTAs overlap
+        // the kernels around them decides between close ones: 64 agents of 62 stations, K = 5, two iterations 2.56 ms
+        // with 2 CTAs per SM and 2.37 ms with 4, equal without it), but for the warm pass, which may follow the
+        // kernel that forms the statistics.
+        bool pdl = false;
         auto hessian_half = [&]() -> cudaError_t {
             cudaError_t err = cudaSuccess;
+            la_hv.pdl = pdl;
             for (int k = 0; k < c->n_cg && err == cudaSuccess; ++k) {
-                if (ssf)
-                    err = launch_ss_sweep(ss_args(c, c->J, c->p, true), true, c->part_hv.grid, c->stream);
-                else
+                if (ssf) {
+                    SSArgs sa = ss_args(c, c->J, c->p, true);
+                    sa.pdl = pdl;
+                    err = launch_ss_sweep(sa, true, c->part_hv.grid, c->stream);
+                } else
                     err = launch_sweep(sweep_args(c, SWEEP_HESSVEC, c->J, c->p), SWEEP_HESSVEC, c->stream);
                 if (err == cudaSuccess) err = launch_cg_step(la_hv, false, c->stream);
             }
@@ -850,14 +858,17 @@ int autotune(calib_ctx* c) {
         };
         auto trial_half = [&]() -> cudaError_t {
             cudaError_t err;
-            if (ssf)
-                err = launch_ss_sweep(ss_args(c, c->J, c->J, false), false, c->part_tr.grid, c->stream);  // J' = J
-            else
+            if (ssf) {
+                SSArgs sa = ss_args(c, c->J, c->J, false);  // J' = J
+                sa.pdl = pdl;
+                err = launch_ss_sweep(sa, false, c->part_tr.grid, c->stream);
+            } else
                 err = launch_sweep(sweep_args(c, SWEEP_TRIAL, c->J, c->x), SWEEP_TRIAL, c->stream);
             return err != cudaSuccess ? err : launch_eval_output(la_tr, c->evOut, c->evL, c->evG, c->stream);
         };
         CK(hessian_half());  // warm
         CK(trial_half());
+        pdl = c->jupdate == CALIB_JUPDATE_LM;
         CK(cudaEventRecord(e0, c->stream));
         for (int r = 0; r < reps; ++r) CK(hessian_half());
         CK(cudaEventRecord(e1, c->stream));
