@@ -52,7 +52,7 @@ NCU_TRAFFIC = {  # dram__bytes_read.sum + dram__bytes_write.sum of one full capt
     ("residual", "fbe001eb534e"): 618.7e6,
 }
 KERNEL_SOURCE = {"sweep_residual": "sweep.cu", "sweep_hessvec": "sweep.cu", "stats_hessvec": "ss_hessvec.cu",
-                 "stats_trial": "ss.cu", "stats_pass": "data.cu", "residual": "data.cu"}
+                 "stats_trial": "ss.cu", "stats_pass": "data.cu", "residual": "data.cu", "jupdate": "jupdate.cu"}
 # The sufficient-statistics passes do 13-17 real flops per algorithmic byte at K=5, above the FP32
 # ridge (~12 flop/B): their roofline is the FP32 pipe. The direct passes are below it (HBM).
 ALU_BOUND = {"stats_hessvec", "stats_trial"}

@@ -228,7 +228,8 @@ int calib_sync(calib_ctx* ctx);
  * stats_trial (sufficient-statistics passes), pcg_step and lm_eval (per-agent LM kernels, no
  * algorithmic byte or flop count: 0), stats_pass (forming the statistics from V and C, timed
  * outside the graph when calib_admm_iter runs it), consensus (the gauge projection, Z-update,
- * Y-update and records of one iteration, timed as one); bytes_per_launch and flops_per_launch are the
+ * Y-update and records of one iteration, timed as one), jupdate (the J-update of small problems, all
+ * its steps in one launch: no byte or flop count); bytes_per_launch and flops_per_launch are the
  * algorithmic bytes and real flops (complex multiply 6, complex multiply-add 8) of one launch.
  * Every output array may be NULL and receives up to cap entries; returns the number of kinds. */
 int calib_profile_enable(calib_ctx* ctx, int on);
@@ -240,8 +241,9 @@ int calib_profile_read(calib_ctx* ctx, int cap, const char** names, double* tota
  * split is CTAs per SM (1, 2, 3, 4, 5, 6, 8, 12, 16, 24) for CALIB_FORM_STATISTICS, chosen per pass,
  * and diagonals per CTA (1, 2, 4, ..., N/2) for CALIB_FORM_DIRECT, one value for both passes (the
  * fastest whole step). calib_admm_iter runs it by itself before its first iteration when the
- * option that fixes the split (ctas_per_sm or chunk_diagonals) is 0; the choice is cached per
- * problem shape for the process. This call re-measures. Outputs (host, any may be NULL): the
+ * option that fixes the split (ctas_per_sm or chunk_diagonals) is 0 and the problem is not so small
+ * that its J-update runs as one launch, which has no split; the choice is cached per problem shape
+ * for the process. This call re-measures. Outputs (host, any may be NULL): the
  * chosen split of the Hessian and of the trial pass, up to cap candidates with the milliseconds of
  * each half, and the candidate count. The iteration state (J, Z, Y) is not changed. */
 int calib_autotune(calib_ctx* ctx, int* split, int* split_trial, int cap, int* candidates,

@@ -30,7 +30,7 @@ __device__ __forceinline__ void report_nonfinite(bool bad, int* status) {
 // the samples, so that a thread's 16-byte accesses are independent and the four samples of a 128-byte line
 // of the source are read one after the other. A reversed pair's V^H takes one entry of each row from the other
 // thread. VEC: the source is 16-byte aligned (else two 8-byte loads). Bound by HBM: 62 stations, 320 agents of 10 samples
-// (388 MB) 76 us with the checks, against 112 + 34 us for an element a thread and a separate pass of checks.
+// (388 MB) 66 us with the checks, against 112 + 34 us for an element a thread and a separate pass of checks.
 constexpr int INGEST_THREADS = 128;
 
 template <bool VEC>
@@ -173,8 +173,8 @@ constexpr int RES_THREADS = 128, RES_SLOTS = 64, RES_T = 2;  // RES_T: samples a
 
 // One CTA per (diagonal, agent), RES_SLOTS slots at a time: first every slot's model matrices M_k = J_ik J_jk^H of the
 // masked directions into shared memory (Ms: [K][2 rows][RES_SLOTS] float4), then the samples, a warp taking
-// 16 slots x 2 samples: 512 contiguous bytes of V a sample and 64 of the output a slot. Bound by HBM:
-// 629 MB (62 stations, K = 5, 320 agents of 10 samples).
+// 16 slots x 2 samples: 512 contiguous bytes of V a sample and 64 of the output a slot. Bound by HBM: 629 MB
+// (62 stations, K = 5, 320 agents of 10 samples) in 136 us, against 205 us with one thread per slot.
 __global__ void __launch_bounds__(RES_THREADS) k_residual(const ResidualArgs a) {
     extern __shared__ __align__(128) unsigned char smem[];
     float4* Ms = reinterpret_cast<float4*>(smem);
@@ -288,9 +288,9 @@ __device__ __forceinline__ float predict_fraction(double turns) {
 // 96 arithmetic instructions (one pair a thread: two 8-byte loads for 6). Phasors of one chunk of sources are formed while the
 // chunk before is summed (two buffers, one barrier a chunk). The sums go through shared memory into the
 // slot layout, so that a slot's directions are written together; long sums are cut into parts there.
-// Measured: 62 stations, 5 directions of 100 sources, 640 (sample, agent)s: 465 us against 760 us with one pair a
-// thread; 20 sources, 3200 (sample, agent)s: 690 against 974 us. What bounds it now is the float64 chain of the
-// turns (37 % of that pipe) beside 6 float32 operations a pair and source (31 % of that pipe).
+// Measured: 62 stations, 5 directions of 100 sources, 640 (sample, agent)s: 418 us against 795 us with one pair a
+// thread (465 us with one CTA of 736 threads an SM, all directions in one group, instead of three CTAs of at most 288).
+// What bounds it is the float64 chain of the turns (37 % of that pipe) beside 6 float32 operations a pair and source (39 %).
 constexpr int PRED_THREADS_SMALL = 288;
 constexpr int PRED_THREADS = 736;  // five directions of 62 stations (720 tiles) at a time; 80 registers
 // Tiles of station blocks delta apart: with the lower block first where some pair of theirs is at most N / 2
