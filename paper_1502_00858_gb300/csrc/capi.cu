@@ -591,8 +591,9 @@ int copy_out(calib_ctx* c, void* dst, const void* dev_src, size_t bytes, int ptr
     return CALIB_OK;
 }
 
+bool aligned(const void* p, size_t bytes) { return reinterpret_cast<uintptr_t>(p) % bytes == 0; }
 // Whether kernels with 16-byte accesses can use a caller's array directly.
-bool usable_in_place(const void* p, int ptr_kind) { return p && ptr_kind == 1 && (reinterpret_cast<uintptr_t>(p) & 15) == 0; }
+bool usable_in_place(const void* p, int ptr_kind) { return p && ptr_kind == 1 && aligned(p, 16); }
 bool overlap(const void* p, size_t np, const void* q, size_t nq) {
     const uintptr_t a = reinterpret_cast<uintptr_t>(p), b = reinterpret_cast<uintptr_t>(q);
     return p && q && a < b + nq && b < a + np;
@@ -1574,7 +1575,8 @@ int calib_eval(calib_ctx* c, const void* Jin, double* L, double* g, void* grad, 
     const size_t ab = (size_t)c->A * sizeof(double);
     const bool apart = !overlap(L, ab, Jin, vb) && !overlap(g, ab, Jin, vb) && !overlap(L, ab, grad, vb) && !overlap(g, ab, grad, vb) &&
                        !overlap(L, ab, g, ab) && (grad == Jin || !overlap(grad, vb, Jin, vb));
-    const bool here = ptr_kind == 1 && apart, grad_here = here && usable_in_place(grad, ptr_kind);
+    // L and g have no alignment but what a copy takes; the kernel's stores want 8 bytes
+    const bool here = ptr_kind == 1 && apart && aligned(L, sizeof(double)) && aligned(g, sizeof(double)), grad_here = here && usable_in_place(grad, ptr_kind);
     CK(cudaMemsetAsync(c->status, 0, sizeof(int), c->stream));
     CK(launch_sweep(sweep_args(c, SWEEP_RESIDUAL, J, nullptr), SWEEP_RESIDUAL, c->stream));
     LMArgs la = lm_args(c, PARTS_DIRECT);
