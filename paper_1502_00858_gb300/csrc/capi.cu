@@ -560,17 +560,17 @@ int stage_in(calib_ctx* c, const void* src, size_t bytes, int ptr_kind, const vo
 }
 
 // Table of a prediction's sources at every frequency, kept with the context up to PREDICT_TABLE bytes. A larger
-// one, and a new one while the stream is being captured or where there is no room, is left out: k_predict
-// then forms the values itself.
+// one, or one where there is no room, is left out: k_predict then forms the values itself. So it does while the
+// stream is being captured: the caller's graph may outlive the table, which a later call replaces by a larger one.
 constexpr size_t PREDICT_TABLE = 64u << 20;
 int predict_workspace(calib_ctx* c, PredictArgs& pa) {
     const size_t want = (size_t)pa.P * pa.K * pa.S * 4 * sizeof(double);
     pa.sources = nullptr;
     if (want > PREDICT_TABLE) return CALIB_OK;
+    cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+    CK(cudaStreamIsCapturing(c->stream, &cap));
+    if (cap != cudaStreamCaptureStatusNone) return CALIB_OK;
     if (want > c->pred_bytes) {
-        cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
-        CK(cudaStreamIsCapturing(c->stream, &cap));
-        if (cap != cudaStreamCaptureStatusNone) return CALIB_OK;
         CK(cudaStreamSynchronize(c->stream));
         cudaFree(c->pred_sources);
         c->pred_sources = nullptr;
