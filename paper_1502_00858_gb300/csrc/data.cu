@@ -175,6 +175,8 @@ constexpr int RES_THREADS = 128, RES_SLOTS = 64, RES_T = 2;  // RES_T: samples a
 // masked directions into shared memory (Ms: [K][2 rows][RES_SLOTS] float4), then the samples, a warp taking
 // 16 slots x 2 samples: 512 contiguous bytes of V a sample and 64 of the output a slot. Bound by HBM: 629 MB
 // (62 stations, K = 5, 320 agents of 10 samples) in 136 us, against 205 us with one thread per slot.
+// VEC: the caller's array is 16-byte aligned (else 8-byte stores, which any complex64 array takes).
+template <bool VEC>
 __global__ void __launch_bounds__(RES_THREADS) k_residual(const ResidualArgs a) {
     extern __shared__ __align__(128) unsigned char smem[];
     float4* Ms = reinterpret_cast<float4*>(smem);
@@ -184,7 +186,7 @@ __global__ void __launch_bounds__(RES_THREADS) k_residual(const ResidualArgs a) 
     const float4* __restrict__ J = reinterpret_cast<const float4*>(a.J) + (size_t)agent * K * N * 2;  // [K][N][2 rows]
     const float4* __restrict__ V = reinterpret_cast<const float4*>(a.V + dsc.voff);                 // [T][n_pad][2 rows]
     const float2* __restrict__ C = a.C + dsc.coff;                                                   // [T][n_pad][K]
-    float4* __restrict__ out = reinterpret_cast<float4*>(a.out + a.vis_off[agent]);                 // [B][T_a][2 rows]
+    float2* __restrict__ out = a.out + a.vis_off[agent];                                            // [B][T_a][2][2]
     for (int g0 = 0; g0 < dsc.n; g0 += RES_SLOTS) {
         const int ng = min(RES_SLOTS, dsc.n - g0);
         __syncthreads();  // the matrices of the slots before are read
@@ -234,9 +236,17 @@ __global__ void __launch_bounds__(RES_THREADS) k_residual(const ResidualArgs a) 
             }
             if (a.correct >= 0) R = mmul(mmul(Li, R), Rj);
             if (rev) R = mherm(R);
-            float4* o = out + ((size_t)b * Ta + t) * 2;
-            o[0] = make_float4(R.e[0][0].x, R.e[0][0].y, R.e[0][1].x, R.e[0][1].y);
-            o[1] = make_float4(R.e[1][0].x, R.e[1][0].y, R.e[1][1].x, R.e[1][1].y);
+            float2* o = out + ((size_t)b * Ta + t) * 4;
+#pragma unroll
+            for (int r = 0; r < 2; ++r) {
+                const cf u = R.e[r][0], w = R.e[r][1];
+                if (VEC) {
+                    *reinterpret_cast<float4*>(o + 2 * r) = make_float4(u.x, u.y, w.x, w.y);
+                } else {
+                    o[2 * r] = make_float2(u.x, u.y);
+                    o[2 * r + 1] = make_float2(w.x, w.y);
+                }
+            }
         }
     }
 }
@@ -610,7 +620,12 @@ cudaError_t launch_extract_coh(const IngestArgs& a, float2* user_dst, cudaStream
     return cudaGetLastError();
 }
 cudaError_t launch_residual(const ResidualArgs& a, cudaStream_t s) {
-    k_residual<<<dim3(a.D, a.A), RES_THREADS, (size_t)a.K * 2 * RES_SLOTS * sizeof(float4), s>>>(a);
+    const dim3 grid(a.D, a.A);
+    const size_t smem = (size_t)a.K * 2 * RES_SLOTS * sizeof(float4);
+    if ((reinterpret_cast<uintptr_t>(a.out) & 15) == 0)
+        k_residual<true><<<grid, RES_THREADS, smem, s>>>(a);
+    else
+        k_residual<false><<<grid, RES_THREADS, smem, s>>>(a);
     return cudaGetLastError();
 }
 // Directions and sources at a time: as many directions as have tiles for the threads, sources to fill the
