@@ -594,29 +594,28 @@ __global__ void __launch_bounds__(BPT == 2 ? LM_MAX_THREADS_BPT2 : LM_MAX_THREAD
 }
 
 // calib_eval: L, g and grad L at a given J (sweep already ran on J), without touching the state. The
-// gradient's terms and the penalty are formed in double-float (df.cuh: float64 operations are slow on this GPU)
-// and the penalty's shares of the threads are added in float64: 34 to 8 us at 320 agents of 310 blocks.
+// gradient's terms and the penalty are formed in float64, which L is returned in: float32's range would not hold the
+// square of a large J - BZ, and double-float holds five bits less. Bound by the float64 rate, hence five operations
+// and five conversions a number: calib_eval at 320 agents of 310 blocks takes 125 us, in double-float it took 119.
 __global__ void __launch_bounds__(EVAL_THREADS) k_eval_output(const LMArgs a, float* grad_out, double* L_out, double* g_out) {
     __shared__ double red[EVAL_THREADS / 32];
     const int agent = blockIdx.x, lane = threadIdx.x & 31, nw = blockDim.x >> 5;
     const int N = a.N, KN = a.K * N;
     const size_t off = (size_t)agent * KN * 8;
-    DF pen{0.f, 0.f};
+    double p = 0.0;
     for (int blk = threadIdx.x; blk < KN; blk += blockDim.x) {
-        const float hr = 0.5f * a.rho[blk / N];
+        const double hr = 0.5 * (double)a.rho[blk / N];
         const Blk gg = sum_parts(a, agent, blk, KN);
         const Blk y = ld_blk(a.Y + off, blk), j = ld_blk(a.Jt + off, blk), bz = ld_blk(a.BZ + off, blk);
         Blk gr;
 #pragma unroll
         for (int i = 0; i < 8; ++i) {
-            const DF d = df_add(DF{j.v[i], 0.f}, DF{-bz.v[i], 0.f});  // exact
-            const DF hd = df_mul(DF{hr, 0.f}, d);                     // rho/2 (J - BZ)
-            gr.v[i] = df_add(df_add(DF{gg.v[i], 0.f}, DF{0.5f * y.v[i], 0.f}), hd).hi;
-            pen = df_add(pen, df_mul(d, df_add(DF{y.v[i], 0.f}, hd)));  // d (y + rho/2 d)
+            const double d = (double)j.v[i] - (double)bz.v[i], yd = y.v[i];
+            gr.v[i] = (float)fma(hr, d, fma(0.5, yd, (double)gg.v[i]));
+            p = fma(d, fma(hr, d, yd), p);  // d (y + rho/2 d)
         }
         st_blk(grad_out + off, blk, gr);
     }
-    double p = df_to_double(pen);
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) p += __shfl_xor_sync(0xffffffffu, p, o);
     if (lane == 0) red[threadIdx.x >> 5] = p;
