@@ -101,7 +101,9 @@ typedef struct {
     int formulation;                   /* CALIB_FORM_STATISTICS (default) or CALIB_FORM_DIRECT */
     int ctas_per_sm;                   /* statistics sweeps: grid = SMs * ctas_per_sm CTAs (at most one
                                           per agent-diagonal), each taking an equal contiguous share of
-                                          the (agent, diagonal) items; 0 = automatic */
+                                          the (agent, diagonal) items; 0 = automatic. A value > 0 also
+                                          keeps small problems on these sweeps, where the automatic
+                                          choice may run their J-update as one launch without them */
     int jupdate;                       /* CALIB_JUPDATE_LM (default), CALIB_JUPDATE_RTR or CALIB_JUPDATE_SAGE */
     int n_sage;                        /* SAGE sweeps per J-update (default 1; CALIB_JUPDATE_SAGE only) */
     int freq_groups;                   /* G >= 1 (default 1; 0 is taken as 1), dividing P: frequency multiplexing. With more
