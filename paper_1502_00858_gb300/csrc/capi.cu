@@ -767,9 +767,10 @@ bool valid_kind(int k) { return k == 0 || k == 1; }
 // Shape class of a tuning result: the timing depends on these alone.
 struct TuneKey {
     int N, K, A, D, form, n_cg;
+    bool pdl;        // how the candidates are launched: as the solver's graph launches them
     long long work;  // total slot-samples (direct form) or slots (statistics)
     bool operator<(const TuneKey& o) const {
-        return std::tie(N, K, A, D, form, n_cg, work) < std::tie(o.N, o.K, o.A, o.D, o.form, o.n_cg, o.work);
+        return std::tie(N, K, A, D, form, n_cg, pdl, work) < std::tie(o.N, o.K, o.A, o.D, o.form, o.n_cg, o.pdl, o.work);
     }
 };
 struct TuneResult { int hv, tr; };  // split of the Hessian and of the trial pass
@@ -798,7 +799,8 @@ int autotune(calib_ctx* c) {
     long long work = 0;
     for (const DiagDesc& d : c->desc_h) work += (long long)d.n;
     for (int a = 0; a < c->A && c->formulation == 1; ++a) work += (long long)c->T[a];
-    const TuneKey key{c->N, c->K, c->A, c->D, c->formulation, c->n_cg, work};
+    const bool lm = c->jupdate == CALIB_JUPDATE_LM;
+    const TuneKey key{c->N, c->K, c->A, c->D, c->formulation, c->n_cg, lm, work};
     auto hit = tune_cache().find(key);
     c->tune_log.clear();
     if (hit != tune_cache().end()) {
@@ -869,7 +871,7 @@ int autotune(calib_ctx* c) {
         };
         CK(hessian_half());  // warm
         CK(trial_half());
-        pdl = c->jupdate == CALIB_JUPDATE_LM;
+        pdl = lm;
         CK(cudaEventRecord(e0, c->stream));
         for (int r = 0; r < reps; ++r) CK(hessian_half());
         CK(cudaEventRecord(e1, c->stream));
