@@ -194,7 +194,7 @@ struct JUpdateArgs {
     int n_lm, n_cg;
     int threads, chunk;  // threads a CTA, diagonals summed at a time
 };
-bool jupdate_plan(int N, int K, int A, int sms, JUpdateArgs& q);  // false: the separate kernels
+bool jupdate_plan(int N, int K, int A, int sms, bool rtr, JUpdateArgs& q);  // false: the separate kernels
 cudaError_t prepare_jupdate_kernels();
 // mode: LM_BEGIN_FROM_PARTIALS or LM_BEGIN_REUSE (LMEvalMode)
 cudaError_t launch_jupdate(const LMArgs& a, const JUpdateArgs& q, bool rtr, int mode, cudaStream_t s);

@@ -1028,7 +1028,7 @@ int calib_init(calib_ctx** out, int n_stations, int n_baselines, const int32_t* 
         return bail(fail(CALIB_ECUDA, "cannot read the SM count"));
     // a caller who fixes the split of the statistics sweeps gets the kernels that have one
     c->one_launch = c->formulation == 0 && opt.ctas_per_sm <= 0 && c->jupdate != CALIB_JUPDATE_SAGE &&
-                    jupdate_plan(N, K, A, c->sms, c->jup);
+                    jupdate_plan(N, K, A, c->sms, c->jupdate == CALIB_JUPDATE_RTR, c->jup);
     if (opt.cuda_stream) {
         c->stream = static_cast<cudaStream_t>(opt.cuda_stream);
     } else {

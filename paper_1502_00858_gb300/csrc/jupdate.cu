@@ -635,16 +635,37 @@ cudaError_t prepare_jupdate_kernels() {
     return e;
 }
 
-bool jupdate_plan(int N, int K, int A, int sms, JUpdateArgs& q) {
+// Whether one launch is the faster one, by the slots (N / 2) N of an agent and the agents an SM has to take. Both sides
+// in us a step of 4 CG steps, separate kernels (autotuned) -> this one, at the edges of the rule (LM unless marked;
+// 8 to 128 stations and 4 to 10240 agents were measured). What a row cites beyond a limit is why the limit lies there.
+//   at most one agent an SM: this one's time does not depend on their number, the separate kernels' grows with it
+//     K = 1: 80 stations, 16 agents 52 -> 44; 96 stations 53 -> 56, but with more than half of the SMs at work every size
+//       (128 stations, 80 agents 96 -> 90, 152: 127 -> 90). Trust region: 80 stations 61 -> 55, 96 59 -> 67
+//     K = 2: 63 stations, 16 agents 58 -> 56. Trust region: 47 stations 62 -> 53, 63 66 -> 75
+//     K = 3: 47 stations, 16 agents 58 -> 53. Trust region: 42 stations 71 -> 65, 44 70 -> 71 (47, 80 agents 80 -> 71)
+//   two (both CTAs resident), 160 agents: K = 1, 80 stations 86 -> 71, 84 84 -> 87; trust region 64 stations 71 -> 55, 80
+//     87 -> 87. 34 stations, K = 2 64 -> 41, K = 3 77 -> 62, trust region 69 -> 59, 85 -> 76
+//   up to eight, or four: K = 1, 80 stations, 320 agents 120 -> 117, 88 139 -> 171; 28 stations, 1200 agents 82 -> 70. 20 stations,
+//     1200 agents, K = 2 91 -> 78, K = 3 127 -> 100. Trust region, 640 agents: 16 stations, K = 1 59 -> 44, K = 3 86 -> 80, K = 2
+//     66 -> 66 (12 stations 68 -> 34); 20 stations, K = 1 65 -> 74; 16 stations, K = 1, 1280 agents 72 -> 73
+//   more: 16 stations, 5120 agents, K = 1 135 -> 127, K = 3 301 -> 246; 20 and 32 stations, K = 1, 2560 agents 112 -> 121 and
+//     137 -> 157, but 33 (where the separate kernels' CTAs grow) 214 -> 183 and 80 681 -> 583; 18 stations, K = 2, 5120
+//     agents 259 -> 289. Trust region: 10 stations, 9600 agents 235 -> 226, 12, 2560 agents 97 -> 99; 16, K = 3 208 -> 200
+bool one_launch_faster(int slots, int K, int A, int sms, bool rtr) {
+    if (A <= sms) {
+        if (2 * A > sms && (rtr ? K == 3 && slots <= 1104 : K == 1)) return true;
+        return slots <= (K == 1 ? 3200 : rtr ? (K == 2 ? 1104 : 900) : K == 2 ? 2048 : 1104);
+    }
+    if (A <= 2 * sms) return slots <= (K == 1 ? (rtr ? 2048 : 3200) : 600);
+    if (A <= (rtr ? 4 : 8) * sms) return slots <= (rtr ? (K == 2 ? 72 : 128) : K == 1 ? 3200 : 200);
+    if (A > 64 * sms) return false;  // not measured
+    if (rtr) return slots <= (K == 3 ? 128 : 50);
+    return slots <= 128 || (K == 1 && slots > 512 && slots <= 3200);
+}
+
+bool jupdate_plan(int N, int K, int A, int sms, bool rtr, JUpdateArgs& q) {
     if (K > 3 || K * N > 512) return false;
-    // Where it is the faster one (10 LM steps x 4 PCG steps, us a step, separate kernels -> this one; one SM works on
-    // an agent, so the separate kernels win back as soon as every SM has many slots):
-    //   K = 1: every size (8 stations 31 -> 14, 62 stations 1280 agents 214 -> 204)
-    //   K = 2, 3: few slots an agent (16 stations, 1280 agents: 103 -> 76 at K = 3), or up to two agents an SM at
-    //   middling ones (32 stations, 320 agents: 82 -> 79; 1280: 176 -> 212), or one agent an SM (47 stations, 64
-    //   agents: 63 -> 53 at K = 3, 160: 87 -> 120; 62 stations 64 agents: 68 -> 56 at K = 2, 76 -> 115 at K = 3).
-    const int slots = (N / 2) * N;
-    if (K > 1 && !(slots <= 200 || (slots <= 600 && A <= 2 * sms) || (A <= sms && slots <= (K == 2 ? 2048 : 1104)))) return false;
+    if (!one_launch_faster(N / 2 * N, K, A, sms, rtr)) return false;
     const size_t fixed = fixed_smem(N, K), diag = diagonal_smem(N, K);
     const int D = N / 2;
     const bool one = A <= sms;  // at most one agent an SM: as many threads as have work
