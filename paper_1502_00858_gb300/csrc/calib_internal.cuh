@@ -259,7 +259,8 @@ struct PredictArgs {
 cudaError_t launch_predict(const PredictArgs& a, cudaStream_t s);
 cudaError_t launch_gram_weights(const float2* C, const DiagDesc* desc, const int* slot, const int* T, float* gw,
                                 int A, int D, int K, int N, cudaStream_t s);
-// Statistics into the full circulant layout and the Jacobi weights (positions of flagged baselines are not written).
+// Statistics into the full circulant layout and, unless gw is NULL, the Jacobi weights (positions of flagged baselines
+// are not written).
 cudaError_t launch_ss_stats(const float2* V, const float2* C, float2* U, float2* S, float* gw, const DiagDesc* desc,
                             const int* slot, const int* T, int A, int D, int K, int N, int Tmax, int* status,
                             cudaStream_t s);

@@ -120,6 +120,8 @@ struct calib_ctx {
     bool one_launch = false;
     JUpdateArgs jup{};
     bool ss_dirty = true;
+    bool gw_dirty = true;      // the Jacobi weights (of C alone) are older than the coherencies
+    bool gw_recorded = false;  // a caller's graph may change the coherencies: the weights are formed every time
     DiagDesc* desc = nullptr;
     int *slot = nullptr, *slot_b = nullptr, *T_d = nullptr;
     int2* flagged = nullptr;  // (agent, baseline) of the flagged baselines
@@ -531,6 +533,7 @@ int build_layout(calib_ctx* c, const uint8_t* flags) {
     c->data_set = false;
     c->coh_set = false;
     c->ss_dirty = true;
+    c->gw_dirty = true;
     return CALIB_OK;
 }
 
@@ -559,6 +562,42 @@ int stage_in(calib_ctx* c, const void* src, size_t bytes, int ptr_kind, const vo
     return CALIB_OK;
 }
 
+// Whether the context's stream is being captured into a caller's graph.
+int recording(calib_ctx* c, bool* cap) {
+    cudaStreamCaptureStatus st = cudaStreamCaptureStatusNone;
+    CK(cudaStreamIsCapturing(c->stream, &st));
+    *cap = st != cudaStreamCaptureStatusNone;
+    return CALIB_OK;
+}
+
+// After the coherencies have changed: their Jacobi weights. The direct form has them formed here, the
+// statistics pass forms them with S.
+int new_coherencies(calib_ctx* c) {
+    bool cap = false;
+    const int rc = recording(c, &cap);
+    if (rc) return rc;
+    if (c->formulation == 1) {
+        CK(launch_gram_weights(c->C, c->desc, c->slot, c->T_d, c->gw, c->A, c->D, c->K, c->N, c->stream));
+        c->launches += 1;
+    }
+    c->gw_dirty = true;
+    c->gw_recorded = c->gw_recorded || cap;
+    c->coh_set = true;
+    return CALIB_OK;
+}
+
+// The statistics of the current data, with the Jacobi weights where the coherencies are new. Visibilities alone leave
+// them as they are, and without them the pass is shorter: 143 to 127 us (62 stations, K = 5, 320 agents of 10 samples),
+// 2029 to 1878 us (K = 10, 1024 agents).
+int statistics_pass(calib_ctx* c) {
+    CK(launch_ss_stats(c->V, c->C, c->ssU, c->ssS, c->gw_dirty || c->gw_recorded ? c->gw : nullptr, c->desc, c->slot, c->T_d, c->A, c->D,
+                       c->K, c->N, c->Tmax, c->status, c->stream));
+    c->launches += 1;
+    c->ss_dirty = false;
+    c->gw_dirty = false;
+    return CALIB_OK;
+}
+
 // Table of a prediction's sources at every frequency, kept with the context up to PREDICT_TABLE bytes. A larger
 // one, or one where there is no room, is left out: k_predict then forms the values itself. So it does while the
 // stream is being captured: the caller's graph may outlive the table, which a later call replaces by a larger one.
@@ -566,10 +605,9 @@ constexpr size_t PREDICT_TABLE = 64u << 20;
 int predict_workspace(calib_ctx* c, PredictArgs& pa) {
     const size_t want = (size_t)pa.P * pa.K * pa.S * 4 * sizeof(double);
     pa.sources = nullptr;
-    if (want > PREDICT_TABLE) return CALIB_OK;
-    cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
-    CK(cudaStreamIsCapturing(c->stream, &cap));
-    if (cap != cudaStreamCaptureStatusNone) return CALIB_OK;
+    bool cap = false;
+    const int rc = recording(c, &cap);
+    if (rc || cap || want > PREDICT_TABLE) return rc;
     if (want > c->pred_bytes) {
         CK(cudaStreamSynchronize(c->stream));
         cudaFree(c->pred_sources);
@@ -1174,11 +1212,8 @@ int calib_set_data(calib_ctx* c, const void* vis, const void* coh, const uint8_t
         ia.is_vis = 0;
         CK(launch_ingest(ia, c->stream));
         c->launches += 1 + (c->n_flagged ? 1 : 0);
-        if (c->formulation == 1) {  // the statistics pass forms the Jacobi weights with S
-            CK(launch_gram_weights(c->C, c->desc, c->slot, c->T_d, c->gw, c->A, c->D, c->K, c->N, c->stream));
-            c->launches += 1;
-        }
-        c->coh_set = true;
+        rc = new_coherencies(c);
+        if (rc) return rc;
     }
     c->data_set = true;
     c->need_eval = true;
@@ -1232,12 +1267,9 @@ int calib_predict(calib_ctx* c, const double* uvw_m, const double* sky, int n_sr
     if (rc) return rc;
     CK(launch_predict(pa, c->stream));
     c->launches += 1 + (pa.sources ? 1 : 0);
-    if (c->formulation == 1) {
-        CK(launch_gram_weights(c->C, c->desc, c->slot, c->T_d, c->gw, c->A, c->D, c->K, c->N, c->stream));
-        c->launches += 1;
-    }
+    rc = new_coherencies(c);
+    if (rc) return rc;
     c->ss_dirty = true;
-    c->coh_set = true;
     c->need_eval = true;
     if (ptr_kind == 0) CK(cudaStreamSynchronize(c->stream));
     return CALIB_OK;
@@ -1364,7 +1396,8 @@ int calib_admm_iter(calib_ctx* c, int n_iters, calib_stats* hist) {
             CK(cudaEventCreate(&p1));
             CK(cudaEventRecord(p0, c->stream));
         }
-        CK(launch_ss_stats(c->V, c->C, c->ssU, c->ssS, c->gw, c->desc, c->slot, c->T_d, c->A, c->D, c->K, c->N, c->Tmax, c->status, c->stream));
+        rc = statistics_pass(c);
+        if (rc) return rc;
         if (c->profiling) {
             CK(cudaEventRecord(p1, c->stream));
             CK(cudaEventSynchronize(p1));
@@ -1375,8 +1408,6 @@ int calib_admm_iter(calib_ctx* c, int n_iters, calib_stats* hist) {
             cudaEventDestroy(p0);
             cudaEventDestroy(p1);
         }
-        c->launches += 1;
-        c->ss_dirty = false;
     }
     if (c->tune_pending && !c->one_launch) {  // the one-launch J-update has no split
         rc = autotune(c);
@@ -1737,9 +1768,8 @@ int calib_autotune(calib_ctx* c, int* split, int* split_trial, int cap, int* can
     if (!c) return fail(CALIB_EINVAL, "ctx is NULL");
     if (!c->data_set || !c->coh_set) return fail(CALIB_ESTATE, "set visibilities and coherencies first");
     if (c->formulation == 0 && c->ss_dirty) {
-        CK(launch_ss_stats(c->V, c->C, c->ssU, c->ssS, c->gw, c->desc, c->slot, c->T_d, c->A, c->D, c->K, c->N, c->Tmax, c->status, c->stream));
-        c->launches += 1;
-        c->ss_dirty = false;
+        const int rs = statistics_pass(c);
+        if (rs) return rs;
     }
     CK(cudaMemsetAsync(c->status, 0, sizeof(int), c->stream));
     tune_cache().clear();

@@ -480,12 +480,13 @@ __global__ void k_gram_weights(const float2* C, const DiagDesc* desc, const int*
 // copies on one mbarrier, so every CTA has its bytes in flight at once; otherwise the samples are
 // read from global memory, two in flight per thread. Written into the full circulant layout:
 // compacted slot g goes to position i = its first station. Positions of flagged baselines are
-// never written (they hold the zeros set when the layout was built). KB >= K: register bucket.
+// never written (they hold the zeros set when the layout was built). KB >= K: register bucket. WEIGHTS: the Jacobi
+// weights too (new coherencies).
 // Largest V + C block staged whole in shared memory; even one CTA per SM keeps far more bytes in
 // flight than the streaming loop.
 constexpr size_t SS_STATS_STAGED_MAX = 200 * 1024;
 
-template <int KB, bool STAGED>
+template <int KB, bool STAGED, bool WEIGHTS>
 __global__ void __launch_bounds__(512, KB > 8 ? 1 : 2) k_ss_stats(const float2* __restrict__ V, const float2* __restrict__ C,
                                                                    float2* __restrict__ U, float2* __restrict__ S,
                                                                    float* __restrict__ gw, int N, const DiagDesc* desc, const int* slot, const int* T,
@@ -566,15 +567,16 @@ __global__ void __launch_bounds__(512, KB > 8 ? 1 : 2) k_ss_stats(const float2* 
 #pragma unroll
         for (int l = 0; l < KB; ++l)
             if (l >= k && l < K) so[l - k] = srow[l];
-        // S_kk is the Jacobi weight of the baseline (see k_gram_weights), at both of its stations
-        float skk = 0.f;
+        if (WEIGHTS) {  // S_kk is the Jacobi weight of the baseline (see k_gram_weights), at both of its stations
+            float skk = 0.f;
 #pragma unroll
-        for (int l = 0; l < KB; ++l)
-            if (l == k) skk = srow[l].x;
-        const int sl = slot[dsc.slot_off + g], f = sl & 0xff, sc = (sl >> 8) & 0xff;
-        float* W = gw + ((size_t)agent * K + k) * N * NP;
-        W[(size_t)f * NP + sc] = skk;
-        W[(size_t)sc * NP + f] = skk;
+            for (int l = 0; l < KB; ++l)
+                if (l == k) skk = srow[l].x;
+            const int sl = slot[dsc.slot_off + g], f = sl & 0xff, sc = (sl >> 8) & 0xff;
+            float* W = gw + ((size_t)agent * K + k) * N * NP;
+            W[(size_t)f * NP + sc] = skk;
+            W[(size_t)sc * NP + f] = skk;
+        }
     }
 }
 
@@ -585,9 +587,12 @@ cudaError_t prepare_data_kernels() {
     const int st = (int)SS_STATS_STAGED_MAX;
     cudaError_t e = cudaFuncSetAttribute(k_predict<PRED_THREADS, 1>, attr, PRED_SMEM_MAX);
     if (e == cudaSuccess) e = cudaFuncSetAttribute(k_predict<PRED_THREADS_SMALL, 3>, attr, PRED_SMEM_MAX);
-    if (e == cudaSuccess) e = cudaFuncSetAttribute(k_ss_stats<4, true>, attr, st);
-    if (e == cudaSuccess) e = cudaFuncSetAttribute(k_ss_stats<8, true>, attr, st);
-    if (e == cudaSuccess) e = cudaFuncSetAttribute(k_ss_stats<MAX_K, true>, attr, st);
+    if (e == cudaSuccess) e = cudaFuncSetAttribute(k_ss_stats<4, true, true>, attr, st);
+    if (e == cudaSuccess) e = cudaFuncSetAttribute(k_ss_stats<8, true, true>, attr, st);
+    if (e == cudaSuccess) e = cudaFuncSetAttribute(k_ss_stats<MAX_K, true, true>, attr, st);
+    if (e == cudaSuccess) e = cudaFuncSetAttribute(k_ss_stats<4, true, false>, attr, st);
+    if (e == cudaSuccess) e = cudaFuncSetAttribute(k_ss_stats<8, true, false>, attr, st);
+    if (e == cudaSuccess) e = cudaFuncSetAttribute(k_ss_stats<MAX_K, true, false>, attr, st);
     return e;
 }
 
@@ -676,10 +681,10 @@ cudaError_t ss_stats_go(const float2* V, const float2* C, float2* U, float2* S, 
                         const int* T, int A, int D, int K, int NP, size_t smem, int* status, cudaStream_t s) {
     const int threads = std::min(512, ((NP * K + 31) / 32) * 32);
     dim3 grid(D, A);
-    if (smem <= SS_STATS_STAGED_MAX)
-        k_ss_stats<KB, true><<<grid, threads, smem, s>>>(V, C, U, S, gw, N, desc, slot, T, D, K, NP, status);
-    else
-        k_ss_stats<KB, false><<<grid, threads, 0, s>>>(V, C, U, S, gw, N, desc, slot, T, D, K, NP, status);
+    const bool staged = smem <= SS_STATS_STAGED_MAX;
+    const auto kernel = staged ? (gw ? k_ss_stats<KB, true, true> : k_ss_stats<KB, true, false>)
+                               : (gw ? k_ss_stats<KB, false, true> : k_ss_stats<KB, false, false>);
+    kernel<<<grid, threads, staged ? smem : 0, s>>>(V, C, U, S, gw, N, desc, slot, T, D, K, NP, status);
     return cudaGetLastError();
 }
 
