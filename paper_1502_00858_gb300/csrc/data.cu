@@ -281,7 +281,7 @@ __global__ void __launch_bounds__(128) k_predict_sources(const PredictArgs a) {
 }
 
 // turns - rint(turns) in float32. The float64 rate is low on this GPU, so the fraction is cut out of the
-// mantissa with integer instructions (64 fractional bits: the same float32 as by rint) from 2^-11 turns on
+// mantissa with integer instructions (64 fractional bits: the same float32 as by rint) from 2^-12 turns on
 // while it has bits there; the rest by rint, in a call, so that it is not executed beside the usual case.
 __device__ __noinline__ float predict_rint_fraction(double turns) { return (float)(turns - rint(turns)); }
 __device__ __forceinline__ float predict_fraction(double turns) {
@@ -289,7 +289,8 @@ __device__ __forceinline__ float predict_fraction(double turns) {
     const int shift = (int)((bits >> 52) & 0x7ff) - 1011;  // |turns| = mantissa 2^(shift - 64)
     if ((unsigned)shift >= 64u) return predict_rint_fraction(turns);
     const long long frac = (long long)((((unsigned long long)bits & 0xfffffffffffffull) | 0x10000000000000ull) << shift);
-    return __ll2float_rn(bits < 0 ? -frac : frac) * 5.421010862427522e-20f;  // 2^-64
+    const float fr = __ll2float_rn(frac) * 5.421010862427522e-20f;  // 2^-64
+    return bits < 0 ? -fr : fr;  // (the integer of one half exactly has no negative)
 }
 
 // One CTA per (sample, agent) and group of directions. The sums c_pq = sum_s I_s E_ps conj(E_qs) are products
