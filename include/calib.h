@@ -35,8 +35,9 @@
  *  - ptr_kind 0: host pointers. The call copies inputs before returning and writes
  *    outputs before returning (it synchronises the library stream).
  *    ptr_kind 1: device pointers, ordered on the library stream (calib_options.cuda_stream).
- *    Device inputs must stay valid until the stream reaches the call; device outputs are
- *    complete once the stream passes the call (calib_sync waits for it).
+ *    Device inputs must stay valid and unchanged until the stream has passed the call (its kernels
+ *    may read them where they are); device outputs are complete then (calib_sync waits for it).
+ *    Device arrays need the alignment of their elements only: 8 bytes for complex64.
  *  - The context owns all of its device memory and frees it in calib_destroy.
  *  - A context is not thread-safe: one thread at a time per context.
  */
@@ -230,8 +231,8 @@ int calib_sync(calib_ctx* ctx);
  * stats_trial (sufficient-statistics passes), pcg_step and lm_eval (per-agent LM kernels, no
  * algorithmic byte or flop count: 0), stats_pass (forming the statistics from V and C, timed
  * outside the graph when calib_admm_iter runs it), consensus (the gauge projection, Z-update,
- * Y-update and records of one iteration, timed as one), jupdate (the J-update of small problems, all
- * its steps in one launch: no byte or flop count); bytes_per_launch and flops_per_launch are the
+ * Y-update and records of one iteration, timed as one), jupdate (the J-update of small problems, all its
+ * steps in one launch: the flops of all its passes, the statistics' bytes once); bytes_per_launch and flops_per_launch are the
  * algorithmic bytes and real flops (complex multiply 6, complex multiply-add 8) of one launch.
  * Every output array may be NULL and receives up to cap entries; returns the number of kinds. */
 int calib_profile_enable(calib_ctx* ctx, int on);
@@ -245,7 +246,8 @@ int calib_profile_read(calib_ctx* ctx, int cap, const char** names, double* tota
  * fastest whole step). calib_admm_iter runs it by itself before its first iteration when the
  * option that fixes the split (ctas_per_sm or chunk_diagonals) is 0 and the problem is not so small
  * that its J-update runs as one launch, which has no split; the choice is cached per problem shape
- * for the process. This call re-measures. Outputs (host, any may be NULL): the
+ * (and per way of launching: dependent launches for LM, plain ones for the other solvers) for the
+ * process. This call re-measures. Outputs (host, any may be NULL): the
  * chosen split of the Hessian and of the trial pass, up to cap candidates with the milliseconds of
  * each half, and the candidate count. The iteration state (J, Z, Y) is not changed. */
 int calib_autotune(calib_ctx* ctx, int* split, int* split_trial, int cap, int* candidates,

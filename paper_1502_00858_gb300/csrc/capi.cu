@@ -498,6 +498,7 @@ int build_layout(calib_ctx* c, const uint8_t* flags) {
     c->TT_res = sweep_tile_samples(smax, K, false);
     c->TT_hv = sweep_tile_samples(smax, K, true);
     if (sweep_threads(smax) > 512) return fail(CALIB_EINVAL, "too many stations for one CTA per diagonal");
+    // (three stages, one more than the sweeps' ring has now: the shapes that are taken stay the same)
     if ((size_t)3 * 24 * 1024 + sweep_smem_bytes(N, K, true) + 4096 > 200 * 1024)
         return fail(CALIB_EINVAL, "N*K too large for the sweep kernels' shared memory");
     if (c->formulation == 0 && ss_sweep_smem_bytes(N, K, false, nullptr) > 200 * 1024)

@@ -301,9 +301,10 @@ __device__ __forceinline__ float predict_fraction(double turns) {
 // slot layout, so that a slot's directions are written together; long sums are cut into parts there.
 // Measured: 62 stations, 5 directions of 100 sources, 640 (sample, agent)s: 418 us against 795 us with one pair a
 // thread (465 us with one CTA of 736 threads an SM, all directions in one group, instead of three CTAs of at most 288).
-// What bounds it is the float64 chain of the turns (37 % of that pipe) beside 6 float32 operations a pair and source (39 %).
-constexpr int PRED_THREADS_SMALL = 288;
-constexpr int PRED_THREADS = 736;  // five directions of 62 stations (720 tiles) at a time; 80 registers
+// No pipe bounds it (float64 37 % busy, FP32 39 %): every warp forms phasors and sums in turn, with one CTA barrier a
+// chunk, and at 72 registers (three CTAs an SM) 88 bytes a thread are spilled.
+constexpr int PRED_THREADS_SMALL = 288;  // up to 288 tiles a direction (62 stations: 144, two directions at a time)
+constexpr int PRED_THREADS = 736;        // more tiles, at most 561 (128 stations); 80 registers, 48 spilled bytes
 // Tiles of station blocks delta apart: with the lower block first where some pair of theirs is at most N / 2
 // apart (held in station order), with the higher block first where some pair is further apart.
 __host__ __device__ inline int predict_tile_fwd(int N, int delta) { return 2 * (delta == 0 ? 1 : 4 * delta - 3) <= N; }
@@ -635,7 +636,7 @@ cudaError_t launch_residual(const ResidualArgs& a, cudaStream_t s) {
     return cudaGetLastError();
 }
 // Directions and sources at a time: as many directions as have tiles for the threads, sources to fill the
-// phasor buffers; the sums of a group use the same shared memory afterwards.
+// phasor buffers; the sums of a group have their own shared memory behind them.
 size_t predict_smem(int N, int KG, int chunk) {
     const size_t N4 = (N + 3) / 4 * 4;
     return (size_t)2 * KG * chunk * (N4 * 8 + 4) / 16 * 16 + 16 + (size_t)(N / 2) * N * KG * 8;

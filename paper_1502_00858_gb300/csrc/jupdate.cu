@@ -2,7 +2,8 @@
 // separate kernels of lm.cu, ss.cu and ss_hessvec.cu spend their time on launches and on chains of dependent
 // loads: all n_lm Levenberg-Marquardt or trust-region steps, each with its n_cg Hessian passes, its CG
 // steps, its trial pass and its accept decision, with the statistics, J, J', the CG direction and the partial
-// sums in shared memory and x, r in registers.
+// sums in shared memory and x, r in registers. (A thread's 128 registers do not hold a whole slot's trial pass at
+// K = 3: 816 bytes are spilled there by the LM form, 656 by the trust region; 36 and 112 at K = 2, none at K = 1.)
 //
 // The arithmetic is that of those kernels, operation by operation: a slot's Q_l, S Q and station terms as in
 // k_ss_hessvec, W, W' and the decrease as in k_ss_sweep, a station's terms summed over the diagonals in
@@ -651,7 +652,7 @@ cudaError_t prepare_jupdate_kernels() {
 //   more: 16 stations, 5120 agents, K = 1 135 -> 127, K = 3 301 -> 246; 20 and 32 stations, K = 1, 2560 agents 112 -> 121 and
 //     137 -> 157, but 33 (where the separate kernels' CTAs grow) 214 -> 183 and 80 681 -> 583; 18 stations, K = 2, 5120
 //     agents 259 -> 289. Trust region: 10 stations, 9600 agents 235 -> 226, 12, 2560 agents 97 -> 99; 16, K = 3 208 -> 200
-bool one_launch_faster(int slots, int K, int A, int sms, bool rtr) {
+static bool one_launch_faster(int slots, int K, int A, int sms, bool rtr) {
     if (A <= sms) {
         if (2 * A > sms && (rtr ? K == 3 && slots <= 1104 : K == 1)) return true;
         return slots <= (K == 1 ? 3200 : rtr ? (K == 2 ? 1104 : 900) : K == 2 ? 2048 : 1104);
