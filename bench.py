@@ -46,10 +46,10 @@ UNIT = "vis*dir*iter/s"
 # DRAM traffic per launch of each sweep kernel from one ncu capture; valid only for the kernel
 # source it was taken on (sha256 prefix of the kernel's .cu file), else reported as null.
 NCU_TRAFFIC = {  # dram__bytes_read.sum + dram__bytes_write.sum of one full capture each (summaries in profiles/)
-    ("stats_hessvec", "effefc092027"): 82.56e6,
-    ("stats_trial", "7102e7ad44aa"): 181.1e6,
-    ("stats_pass", "fbe001eb534e"): 592.6e6,
-    ("residual", "fbe001eb534e"): 618.7e6,
+    ("stats_hessvec", "effefc092027"): 82.02e6,
+    ("stats_trial", "8c09e6c550b8"): 180.9e6,
+    ("stats_pass", "708731329d50"): 622.4e6,
+    ("residual", "708731329d50"): 623.5e6,
 }
 KERNEL_SOURCE = {"sweep_residual": "sweep.cu", "sweep_hessvec": "sweep.cu", "stats_hessvec": "ss_hessvec.cu",
                  "stats_trial": "ss.cu", "stats_pass": "data.cu", "residual": "data.cu", "jupdate": "jupdate.cu"}

@@ -301,8 +301,9 @@ __device__ __forceinline__ float predict_fraction(double turns) {
 // slot layout, so that a slot's directions are written together; long sums are cut into parts there.
 // Measured: 62 stations, 5 directions of 100 sources, 640 (sample, agent)s: 418 us against 795 us with one pair a
 // thread (465 us with one CTA of 736 threads an SM, all directions in one group, instead of three CTAs of at most 288).
-// No pipe bounds it (float64 37 % busy, FP32 39 %): every warp forms phasors and sums in turn, with one CTA barrier a
-// chunk, and at 72 registers (three CTAs an SM) 88 bytes a thread are spilled.
+// No pipe bounds it (float64 46 % busy, FP32 38 %, issue 62 %): every warp forms phasors and sums in turn, with one CTA
+// barrier a chunk, half of the shared wavefronts are bank conflicts, and at 72 registers (three CTAs an SM) 88 bytes
+// a thread are spilled.
 constexpr int PRED_THREADS_SMALL = 288;  // up to 288 tiles a direction (62 stations: 144, two directions at a time)
 constexpr int PRED_THREADS = 736;        // more tiles, at most 561 (128 stations); 80 registers, 48 spilled bytes
 // Tiles of station blocks delta apart: with the lower block first where some pair of theirs is at most N / 2
